@@ -320,7 +320,11 @@ hvx_status hvxSetGraphFusion(hvx_graph g, int32_t enable);
  * the same); HVX_CODEGEN_COLS=4 turns on 4-column blocks (vector loads
  * and stores) in the output pass of 128-wide tiles (slower on the
  * applications measured; kept for experiments);
- * HVX_CODEGEN_VERBOSE=1 prints why a group got no generated kernel. */
+ * HVX_CODEGEN_VERBOSE=1 prints why a group got no generated kernel.  Groups
+ * of U8 / S16 / UYVY images whose sums fit 16 bits run a second form of the
+ * kernel (pixel pairs in 16-bit lanes, strips of 8 columns x R rows per
+ * thread); HVX_STRIP_ROWS=R overrides R, and 0 or any HVX_CODEGEN_TMA / ROWS /
+ * COLS / MINBLOCKS setting keeps the tile form. */
 hvx_status hvxSetGraphCodegen(hvx_graph g, int32_t mode);
 
 /* Source text of the kernel generated for launch `group` of a verified graph

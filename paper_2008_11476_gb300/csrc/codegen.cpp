@@ -19,6 +19,10 @@
 //     validity or fill test; the others run the checked instance of the same
 //     template.
 // Kernels are cached by source text, so graphs of the same shape share one.
+// A group whose images fit 16-bit lanes runs the strip form instead
+// (codegen_strip.cpp, faster at every size measured); the tile form stays for
+// S32 / F32 images, 64-bit user operators, global operators and sums beyond 16
+// bits, and for the tuning knobs that ask for one of its variants.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <dlfcn.h>
@@ -37,6 +41,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "codegen_strip.h"
 #include "hvx_internal.h"
 #include "jit_params.h"
 #include "kernel_params.h"
@@ -67,6 +72,7 @@ typedef CUresult (*FnModuleGetFunction)(CUfunction*, CUmodule, const char*);
 typedef CUresult (*FnFuncSetAttribute)(CUfunction, CUfunction_attribute, int);
 typedef CUresult (*FnLaunchKernel)(CUfunction, unsigned, unsigned, unsigned, unsigned, unsigned,
                                    unsigned, unsigned, CUstream, void**, void**);
+typedef CUresult (*FnOccupancy)(int*, CUfunction, int, size_t);
 typedef CUresult (*FnLaunchKernelEx)(const CUlaunchConfig*, CUfunction, void**, void**);
 
 struct Nvrtc {
@@ -119,6 +125,7 @@ struct Driver {
     FnModuleGetFunction get = nullptr;
     FnFuncSetAttribute attr = nullptr;
     FnLaunchKernel launch = nullptr;
+    FnOccupancy occupancy = nullptr;
     FnLaunchKernelEx launch_ex = nullptr;  // optional: programmatic dependent launches
 };
 
@@ -141,8 +148,9 @@ Driver& driver() {
         d.get = (FnModuleGetFunction)entry("cuModuleGetFunction");
         d.attr = (FnFuncSetAttribute)entry("cuFuncSetAttribute");
         d.launch = (FnLaunchKernel)entry("cuLaunchKernel");
+        d.occupancy = (FnOccupancy)entry("cuOccupancyMaxActiveBlocksPerMultiprocessor");
         d.launch_ex = (FnLaunchKernelEx)entry("cuLaunchKernelEx");
-        d.ok = d.load && d.get && d.attr && d.launch;
+        d.ok = d.load && d.get && d.attr && d.launch && d.occupancy;
     });
     return d;
 }
@@ -161,6 +169,15 @@ struct JitKernel {
     CUfunction fn_batch = nullptr;  // several images per launch
     int smem_bytes = 0;
     int tw = 0, th = 0;
+    std::vector<std::array<int, 3>> tma_boxes;  // tile form: (input, width, height)
+    // the strip form (codegen_strip.cpp): compiled and run instead of the tile
+    // form where the group has one
+    bool strips = false;
+    StripPlan strip;
+    // the group's images: halo, and whether it is an external input
+    int n_buf = 0;
+    std::array<int, HVX_JIT_MAX_BUF> halo{};
+    std::array<bool, HVX_JIT_MAX_BUF> is_in{};
 };
 
 namespace {
@@ -169,6 +186,7 @@ namespace {
 // Source emission
 
 constexpr int kThreads = 256;  // 8 warps: warps take rows, lanes columns
+constexpr int kStripSmem = 110 * 1024;  // most shared memory of a strip tile
 
 struct Emitter {
     const GenericDesc& d;
@@ -212,7 +230,13 @@ struct Emitter {
     Emitter(const GenericDesc& desc, const std::vector<std::string>& u) : d(desc), user(u) {
         const char* env = std::getenv("HVX_CODEGEN_TMA");
         tma = !(env && env[0] == '0');
+        for (const char* n : {"HVX_CODEGEN_TMA", "HVX_CODEGEN_ROWS", "HVX_CODEGEN_COLS",
+                              "HVX_CODEGEN_MINBLOCKS"})
+            tile_knobs = tile_knobs || std::getenv(n);
+        const char* rows = std::getenv("HVX_STRIP_ROWS");
+        tile_knobs = tile_knobs || (rows && std::atoi(rows) == 0);
     }
+    bool tile_knobs = false;         // a tuning knob of the tile form is set: no strip form
     bool tma = true;                 // stage U8 inputs of interior tiles by TMA
     std::vector<int> load_bar;       // per pass: word offset of its mbarrier, or -1
 
@@ -1409,6 +1433,8 @@ struct Emitter {
           << "      const long long c1 = clock64();\n"
           << "      while (!hvx_mbar_try(bar) && clock64() - c1 < (1ll << 31)) {}\n"
           << "      return;\n    }\n  }\n}\n\n"
+          << "// ---- tile form; not compiled where the group has a strip form (below) ----\n"
+          << "#ifndef HVX_STRIPS\n"
           << "template <bool CHECK, bool GMAP>\n"
           << "__device__ __forceinline__ void hvx_tile(const HvxJitParams& p, int* smem, int x0, "
              "int y0) {\n"
@@ -1513,7 +1539,7 @@ struct Emitter {
           << "    hvx_tile<false, true>(p, smem, tx * " << tw << ", ty * " << th << ");\n"
           << "  else\n"
           << "    hvx_tile<true, true>(p, smem, tx * " << tw << ", ty * " << th << ");\n"
-          << "}\n";
+          << "}\n#endif\n";
         return true;
     }
 };
@@ -1544,8 +1570,8 @@ bool compile(JitKernel& k) {
     }
     // no fast-math flags: the exact arithmetic relies on IEEE division and sqrt
     const char* opts[] = {"--gpu-architecture=sm_103a", "--std=c++17", "--device-int128",
-                          "-default-device"};
-    const int r = n.compile(prog, 4, opts);
+                          "-default-device", "-DHVX_STRIPS"};
+    const int r = n.compile(prog, k.strips ? 5 : 4, opts);
     size_t ls = 0;
     if (n.log_size(prog, &ls) == 0 && ls > 1) {
         k.log.assign(ls, '\0');
@@ -1570,15 +1596,16 @@ bool load(JitKernel& k, int device, std::string* why) {
         return false;
     }
     if (dr.load(&k.mod, k.cubin.data()) != CUDA_SUCCESS ||
-        dr.get(&k.fn, k.mod, "hvx_generated") != CUDA_SUCCESS ||
-        dr.get(&k.fn_batch, k.mod, "hvx_generated_batch") != CUDA_SUCCESS) {
+        dr.get(&k.fn, k.mod, k.strips ? "hvx_generated_strips" : "hvx_generated") != CUDA_SUCCESS ||
+        dr.get(&k.fn_batch, k.mod,
+               k.strips ? "hvx_generated_strips_batch" : "hvx_generated_batch") != CUDA_SUCCESS) {
         *why = "cuModuleLoadData / cuModuleGetFunction failed";
         return false;
     }
-    if (k.smem_bytes > 48 * 1024 &&
-        (dr.attr(k.fn, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, k.smem_bytes) !=
-             CUDA_SUCCESS ||
-         dr.attr(k.fn_batch, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, k.smem_bytes) !=
+    const int smem = k.strips ? kStripSmem : k.smem_bytes;
+    if (smem > 48 * 1024 &&
+        (dr.attr(k.fn, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, smem) != CUDA_SUCCESS ||
+         dr.attr(k.fn_batch, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, smem) !=
              CUDA_SUCCESS)) {
         *why = "cuFuncSetAttribute failed";
         return false;
@@ -1594,33 +1621,176 @@ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 bool jit_available() { return nvrtc().ok; }
 
-bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code, bool load_module,
-                 int device, JitLaunch* out, std::string* why) {
+namespace {
+
+// Interior tiles and grid of a launch: every image's cells of an interior
+// tile grown by its halo lie in its valid region (external inputs: in the
+// image; they are read as stored).  p.rows = 0 is the tile form.  Returns the
+// bytes of shared memory.
+int set_tiles(const JitKernel& k, HvxJitParams& p, unsigned* gx, unsigned* gy) {
+    const int tw = p.rows ? STRIP_TW : k.tw, th = p.rows ? 8 * p.rows : k.th;
+    *gx = (unsigned)((p.W + tw - 1) / tw);
+    *gy = (unsigned)((p.H + th - 1) / th);
+    int ix0 = 0, iy0 = 0, ix1 = (int)*gx - 1, iy1 = (int)*gy - 1;
+    for (int b = 0; b < k.n_buf; ++b) {
+        const int h = k.halo[b];
+        int r[4] = {0, 0, p.W, p.H};
+        if (!k.is_in[b])
+            for (int i = 0; i < 4; ++i) r[i] = p.valid[b][i];
+        ix0 = std::max(ix0, ceil_div(r[0] + h, tw));
+        iy0 = std::max(iy0, ceil_div(r[1] + h, th));
+        ix1 = std::min(ix1, floor_div(r[2] - h - tw, tw));
+        iy1 = std::min(iy1, floor_div(r[3] - h - th, th));
+    }
+    p.ix0 = ix0;
+    p.ix1 = ix1;
+    p.iy0 = iy0;
+    p.iy1 = iy1;
+    return p.rows ? strip_smem_bytes(k.strip, p.rows) : k.smem_bytes;
+}
+
+// Tensor maps of the inputs that the launch's form stages by TMA.
+bool set_maps(const JitKernel& k, HvxJitParams& p) {
+    static_assert(sizeof(HvxTensorMap) == sizeof(CUtensorMap), "tensor map blob");
+    auto encode = [&](int e, int elem, int bw, int bh) {
+        return encode_map_raw(reinterpret_cast<CUtensorMap*>(&p.tmap[e]), p.in[e], p.in_pitch[e],
+                              (uint32_t)p.W, (uint32_t)p.H, (uint32_t)bw, (uint32_t)bh, elem) ==
+               HVX_SUCCESS;
+    };
+    if (p.rows) {
+        for (const StripBox& b : k.strip.boxes)
+            if (!encode(b.ext, b.elem, STRIP_BOX_W, 8 * p.rows + 2 * b.halo)) return false;
+    } else {
+        for (const auto& b : k.tma_boxes)
+            if (!encode(b[0], 1, b[1], b[2])) return false;
+    }
+    return true;
+}
+
+// Rows per thread of a strip launch over n images.  A CTA's time grows with
+// its R rows and the prologue steps before them; the launch takes waves of the
+// CTAs that are resident at a time (registers, and boxes that grow with R), the
+// last one partly filled.  Minimising max(1, waves + 1/2) (R + 0.3 prologue +
+// 1) comes within 0.4 % of the best R in the mean and 5.5 % at worst over 44
+// measured points (FChain, Unsharp, Laplacian and a morphology graph; 64x48 to
+// 3840x2160; 1 to 16 frames; R = 3 .. 24): small launches want R = 3 (1080p
+// Unsharp frame: 5.0 us, 11.8 at R = 15), 16 x 1080p FChain R = 15 (57 us, 107
+// at R = 3), 16 x 1080p Unsharp R = 9 (25 us, 41 and 40 at R = 3 and 24).
+// HVX_STRIP_ROWS in the environment overrides (0: the tile form).
+int strip_rows(const JitKernel& k, const int* W, const int* H, int n, int num_sms) {
+    const int u = k.strip.unroll;
+    if (const char* e = getenv("HVX_STRIP_ROWS")) {
+        const int r = atoi(e);
+        if (r >= u && r <= 24) return r / u * u;
+    }
+    int pro = 0;
+    for (int b = 0; b < k.n_buf; ++b) pro = std::max(pro, 2 * k.halo[b]);
+    int best = u;
+    double best_cost = 1e30;
+    for (int r = u; r <= 24; r += u) {
+        const int smem = strip_smem_bytes(k.strip, r);
+        if (smem > kStripSmem) break;
+        int per = 5;
+        if (k.fn_batch && driver().occupancy(&per, k.fn_batch, STRIP_THREADS, (size_t)smem) !=
+                              CUDA_SUCCESS)
+            per = 5;
+        long long tiles = 0;
+        for (int i = 0; i < n; ++i)
+            tiles += (long long)((W[i] + STRIP_TW - 1) / STRIP_TW) * ((H[i] + 8 * r - 1) / (8 * r));
+        const double waves = (double)tiles / ((double)std::max(per, 1) * num_sms);
+        const double cost = std::max(1.0, waves + 0.5) * (r + 0.3 * pro + 1.0);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = r;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
+namespace {
+
+// Everything of a group that its generated source depends on (not sizes,
+// addresses or pitches), so that graphs of a known shape skip the emission.
+std::string shape_key(const GenericDesc& d, const std::vector<std::string>& user, int device) {
+    GenericDesc c;
+    std::memcpy(&c, &d, sizeof(c));  // (zero-initialised by the planner, padding included)
+    for (int b = 0; b < c.n_buf; ++b) {
+        int32_t* v = c.buf[b].valid;
+        v[0] = v[0] == 0 && v[1] == 0 && v[2] == c.W && v[3] == c.H;
+        v[1] = v[2] = v[3] = 0;
+    }
+    c.W = c.H = 0;
+    for (int e = 0; e < GEN_MAX_EXT; ++e) {
+        c.in[e].ptr = c.out[e].ptr = nullptr;
+        c.in[e].pitch = c.out[e].pitch = 0;
+    }
+    for (int k = 0; k < c.n_stage; ++k) c.st[k].res = nullptr;
+    std::string key(reinterpret_cast<const char*>(&c), sizeof(c));
+    key += std::to_string(device);
+    for (const char* n : {"HVX_CODEGEN_TMA", "HVX_CODEGEN_ROWS", "HVX_CODEGEN_COLS",
+                          "HVX_CODEGEN_MINBLOCKS", "HVX_STRIP_ROWS"}) {
+        const char* v = std::getenv(n);
+        key += '\n';
+        if (v) key += std::string("=") + v;
+    }
+    for (const std::string& u : user) key += '\n' + u;
+    return key;
+}
+
+// The kernel of a group, emitted and compiled if no graph of its shape has
+// been prepared yet (g_mu is held).
+JitKernel* find_kernel(const GenericDesc& d, const std::vector<std::string>& user_code, int device,
+                       std::string* why) {
+    static auto* by_shape = new std::unordered_map<std::string, JitKernel*>();
+    const std::string shape = shape_key(d, user_code, device);
+    auto it = by_shape->find(shape);
+    if (it != by_shape->end()) return it->second;
     Emitter em(d, user_code);
     if (!em.emit()) {
         *why = "group shape not handled by the code generator";
-        return false;
+        return nullptr;
     }
-    const std::string src = em.o.str();
+    std::string src = em.o.str(), strip_src;
+    StripPlan strip;
+    const bool strips = !em.tile_knobs && emit_strips(d, &strip_src, &strip);
+    if (strips) src += strip_src;
+    std::unique_ptr<JitKernel>& slot = cache()[std::to_string(device) + "\n" + src];
+    if (!slot) {
+        slot.reset(new JitKernel);
+        slot->source = src;
+        slot->tw = em.tw;
+        slot->th = em.th;
+        slot->smem_bytes = em.smem_words * 4;
+        slot->tma_boxes = em.tma_boxes();
+        slot->strips = strips;
+        slot->strip = strip;
+        slot->n_buf = d.n_buf;
+        for (int b = 0; b < d.n_buf; ++b) {
+            slot->halo[b] = d.buf[b].halo;
+            slot->is_in[b] = em.ext_in[b] >= 0;
+        }
+        compile(*slot);
+    }
+    (*by_shape)[shape] = slot.get();
+    return slot.get();
+}
+
+}  // namespace
+
+bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code, bool load_module,
+                 int device, JitLaunch* out, std::string* why) {
     JitKernel* k = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_mu);
-        std::unique_ptr<JitKernel>& slot =
-            cache()[(load_module ? std::to_string(device) : std::string("-")) + "\n" + src];
-        if (!slot) {
-            slot.reset(new JitKernel);
-            slot->source = src;
-            slot->tw = em.tw;
-            slot->th = em.th;
-            slot->smem_bytes = em.smem_words * 4;
-            compile(*slot);
-        }
-        if (!slot->compiled) {
-            *why = "NVRTC: " + slot->log;
+        k = find_kernel(d, user_code, load_module ? device : -1, why);
+        if (!k) return false;
+        if (!k->compiled) {
+            *why = "NVRTC: " + k->log;
             return false;
         }
-        if (load_module && slot->device != device && !load(*slot, device, why)) return false;
-        k = slot.get();
+        if (load_module && k->device != device && !load(*k, device, why)) return false;
     }
     JitLaunch& j = *out;
     j.k = k;
@@ -1644,83 +1814,100 @@ bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code
             if (nres >= HVX_JIT_MAX_RES) return false;
             p.res[nres++] = d.st[k].res;
         }
-    // interior tiles: every image's cells of the tile grown by its halo lie in
-    // its valid region (external inputs: in the image; they are read as stored)
-    const int tw = k->tw, th = k->th;
-    j.gx = (unsigned)((d.W + tw - 1) / tw);
-    j.gy = (unsigned)((d.H + th - 1) / th);
-    int ix0 = 0, iy0 = 0, ix1 = (int)j.gx - 1, iy1 = (int)j.gy - 1;
-    std::vector<bool> is_in(d.n_buf, false);
-    for (int e = 0; e < d.n_in; ++e) is_in[d.in[e].buf] = true;
-    for (int b = 0; b < d.n_buf; ++b) {
-        const int h = d.buf[b].halo;
-        int r[4] = {0, 0, (int)d.W, (int)d.H};
-        if (!is_in[b])
-            for (int i = 0; i < 4; ++i) r[i] = d.buf[b].valid[i];
-        ix0 = std::max(ix0, ceil_div(r[0] + h, tw));
-        iy0 = std::max(iy0, ceil_div(r[1] + h, th));
-        ix1 = std::min(ix1, floor_div(r[2] - h - tw, tw));
-        iy1 = std::min(iy1, floor_div(r[3] - h - th, th));
+    int num_sms = 152;
+    if (load_module) cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
+    const int rows = k->strips ? strip_rows(*k, &d.W, &d.H, 1, num_sms) : 0;
+    p.rows = rows;
+    j.smem = set_tiles(*k, p, &j.gx, &j.gy);
+    if (load_module && !set_maps(*k, p)) {
+        *why = "tensor map of a staged input";
+        return false;
     }
-    p.ix0 = ix0;
-    p.ix1 = ix1;
-    p.iy0 = iy0;
-    p.iy1 = iy1;
-    // tensor maps of the TMA-staged inputs (box = the input's slot)
-    static_assert(sizeof(HvxTensorMap) == sizeof(CUtensorMap), "tensor map blob");
-    if (load_module)
-        for (const auto& bx : em.tma_boxes()) {
-            const GenExt& in = d.in[bx[0]];
-            if (encode_u8_map_raw(reinterpret_cast<CUtensorMap*>(&p.tmap[bx[0]]), in.ptr, in.pitch,
-                                  (uint32_t)d.W, (uint32_t)d.H, (uint32_t)bx[1],
-                                  (uint32_t)bx[2]) != HVX_SUCCESS) {
-                *why = "tensor map of a staged input";
-                return false;
-            }
-        }
     return true;
 }
 
+namespace {
+
+// A launch with programmatic stream serialisation: it may begin while the
+// previous kernel on the stream finishes (the kernel waits for it).
+CUresult launch_dependent(CUfunction fn, unsigned gx, unsigned gy, unsigned gz, unsigned threads,
+                          int smem, cudaStream_t s, void** args) {
+    const Driver& dr = driver();
+    if (!dr.launch_ex)
+        return dr.launch(fn, gx, gy, gz, threads, 1, 1, (unsigned)smem, (CUstream)s, args, nullptr);
+    CUlaunchAttribute attr = {};
+    attr.id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
+    attr.value.programmaticStreamSerializationAllowed = 1;
+    CUlaunchConfig cfg = {};
+    cfg.gridDimX = gx;
+    cfg.gridDimY = gy;
+    cfg.gridDimZ = gz;
+    cfg.blockDimX = threads;
+    cfg.blockDimY = 1;
+    cfg.blockDimZ = 1;
+    cfg.sharedMemBytes = (unsigned)smem;
+    cfg.hStream = (CUstream)s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return dr.launch_ex(&cfg, fn, args, nullptr);
+}
+
+}  // namespace
+
 cudaError_t jit_launch(const JitLaunch& j, cudaStream_t s) {
     void* args[] = {const_cast<HvxJitParams*>(&j.p)};
-    const Driver& dr = driver();
-    CUresult r;
-    if (dr.launch_ex) {
-        // programmatic stream serialisation: the launch may begin while the
-        // previous kernel on the stream finishes (the kernel waits for it)
-        CUlaunchAttribute attr = {};
-        attr.id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
-        attr.value.programmaticStreamSerializationAllowed = 1;
-        CUlaunchConfig cfg = {};
-        cfg.gridDimX = j.gx;
-        cfg.gridDimY = j.gy;
-        cfg.gridDimZ = 1;
-        cfg.blockDimX = kThreads;
-        cfg.blockDimY = 1;
-        cfg.blockDimZ = 1;
-        cfg.sharedMemBytes = (unsigned)j.k->smem_bytes;
-        cfg.hStream = (CUstream)s;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        r = dr.launch_ex(&cfg, j.k->fn, args, nullptr);
-    } else {
-        r = dr.launch(j.k->fn, j.gx, j.gy, 1, kThreads, 1, 1, (unsigned)j.k->smem_bytes,
-                      (CUstream)s, args, nullptr);
+    return launch_dependent(j.k->fn, j.gx, j.gy, 1, j.p.rows ? STRIP_THREADS : kThreads, j.smem, s,
+                            args) == CUDA_SUCCESS
+               ? cudaSuccess
+               : cudaErrorLaunchFailure;
+}
+
+hvx_status jit_batch_params(const JitLaunch* const* js, int n, int num_sms, HvxJitParams* out,
+                            int* tiles, JitBatch* b) {
+    const JitKernel& k = *js[0]->k;
+    std::vector<int> W(n), H(n);
+    for (int i = 0; i < n; ++i) {
+        W[i] = js[i]->p.W;
+        H[i] = js[i]->p.H;
     }
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
+    const int rows = k.strips ? strip_rows(k, W.data(), H.data(), n, num_sms) : 0;
+    long long total = 0;
+    for (int i = 0; i < n; ++i) {
+        HvxJitParams& p = out[i];
+        p = js[i]->p;
+        p.rows = rows;
+        unsigned gx = 0, gy = 0;
+        b->smem = set_tiles(k, p, &gx, &gy);
+        tiles[i] = (int)(gx * gy);
+        total += tiles[i];
+        if (!set_maps(k, p)) return HVX_ERROR_DEVICE;
+    }
+    if (total > (1ll << 30)) return HVX_ERROR_NOT_SUPPORTED;
+    b->k = js[0]->k;
+    b->n = n;
+    b->rows = rows;
+    b->gx = (unsigned)total;
+    b->gy = b->gz = 1;
+    bool same = rows > 0 && n <= 65535;
+    for (int i = 1; i < n; ++i) same = same && W[i] == W[0] && H[i] == H[0];
+    b->uniform = same;
+    if (same) {
+        b->gx = (unsigned)((W[0] + STRIP_TW - 1) / STRIP_TW);
+        b->gy = (unsigned)((H[0] + 8 * rows - 1) / (8 * rows));
+        b->gz = (unsigned)n;
+    }
+    return HVX_SUCCESS;
 }
 
-cudaError_t jit_launch_batch(const JitKernel* k, const HvxJitParams* params, const int* tile_start,
-                             int n, int total_tiles, cudaStream_t s) {
-    void* args[] = {&params, &tile_start, &n};
-    const CUresult r = driver().launch(k->fn_batch, (unsigned)total_tiles, 1, 1, kThreads, 1, 1,
-                                       (unsigned)k->smem_bytes, (CUstream)s, args, nullptr);
+cudaError_t jit_launch_batch(const JitBatch& b, const HvxJitParams* params, const int* tile_start,
+                             cudaStream_t s) {
+    int n = b.n, rows = b.uniform ? b.rows : 0;
+    void* args[] = {&params, &tile_start, &n, &rows};  // the tile form takes the first three
+    const CUresult r =
+        b.rows ? launch_dependent(b.k->fn_batch, b.gx, b.gy, b.gz, STRIP_THREADS, b.smem, s, args)
+               : driver().launch(b.k->fn_batch, b.gx, b.gy, b.gz, kThreads, 1, 1,
+                                 (unsigned)b.smem, (CUstream)s, args, nullptr);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
-}
-
-void jit_tile(const JitKernel* k, int* tw, int* th) {
-    *tw = k->tw;
-    *th = k->th;
 }
 
 const std::string& jit_source(const JitLaunch& j) { return j.k->source; }

@@ -199,8 +199,9 @@ inline bool border_wraps(int border) {
 struct JitKernel;
 struct JitLaunch {
     JitKernel* k = nullptr;  // cached for the life of the process
-    HvxJitParams p;
+    HvxJitParams p;  // p.rows > 0: the strip form
     unsigned gx = 0, gy = 0;
+    int smem = 0;
 };
 
 // A fused group: ops run by one kernel launch.
@@ -315,10 +316,10 @@ hvx_status check_device_error(Context* ctx);
 hvx_status ensure_context_device_state(Context* ctx);
 void destroy_batch_cache(Context* ctx);
 hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s);
-// 2-D U8 tensor map of (w x h) bytes at ptr (16-byte aligned, pitch a multiple
+// 2-D tensor map of (w x h) elements of 1 or 2 bytes at ptr (16-byte aligned, pitch a multiple
 // of 16) with a (box_w x box_h) box; cells outside the image read as 0.
-hvx_status encode_u8_map_raw(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
-                             uint32_t h, uint32_t box_w, uint32_t box_h);
+hvx_status encode_map_raw(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
+                          uint32_t h, uint32_t box_w, uint32_t box_h, int elem_bytes);
 // The tuned launch of a cached batch of exactly these graphs: rows per thread
 // of each image's tiles (0 where the kernel has its own tile) and the
 // persistent grid (0 for a direct launch).  HVX_ERROR_INVALID_PARAMETERS when
@@ -336,11 +337,21 @@ bool jit_available();
 bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code, bool load_module,
                  int device, JitLaunch* out, std::string* why);
 cudaError_t jit_launch(const JitLaunch& j, cudaStream_t s);
-// n images' groups that run the same generated kernel, in one launch: params
-// and tile_start (n + 1 prefix sums of tiles per image) in device memory
-cudaError_t jit_launch_batch(const JitKernel* k, const HvxJitParams* params, const int* tile_start,
-                             int n, int total_tiles, cudaStream_t s);
-void jit_tile(const JitKernel* k, int* tw, int* th);
+// n images' groups that run the same generated kernel, in one launch: their
+// parameters (host copies, the form and its rows chosen for the whole batch)
+// and tile counts, then the launch with params and tile_start (n + 1 prefix
+// sums of tiles per image) in device memory
+struct JitBatch {
+    JitKernel* k = nullptr;
+    int n = 0, smem = 0;
+    int rows = 0;          // > 0: the strip form
+    bool uniform = false;  // strips of images of one size: grid (tiles x, tiles y, images)
+    unsigned gx = 0, gy = 1, gz = 1;
+};
+hvx_status jit_batch_params(const JitLaunch* const* js, int n, int num_sms, HvxJitParams* out,
+                            int* tiles, JitBatch* b);
+cudaError_t jit_launch_batch(const JitBatch& b, const HvxJitParams* params, const int* tile_start,
+                             cudaStream_t s);
 const std::string& jit_source(const JitLaunch& j);
 
 // host data of a call (api.cpp): checks, and the 2-D copies in one direction

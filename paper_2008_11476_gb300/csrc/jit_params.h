@@ -26,5 +26,7 @@ struct HvxJitParams {
     unsigned long long out_pitch[HVX_JIT_MAX_EXT];
     void* res[HVX_JIT_MAX_RES];     // result blocks of the group's global operators
     int* err;                       // device error word (a bounded wait that ran out)
-    HvxTensorMap tmap[HVX_JIT_MAX_EXT];  // U8 inputs staged by TMA: box = the staged slot
+    int rows;                       // strip form: output rows per thread (tiles of 128 x 8 rows)
+    HvxTensorMap tmap[HVX_JIT_MAX_EXT];  // inputs staged by TMA: box = the staged slot (tile
+                                         // form) or 160 x (8 rows + 2 halo) pixels (strip form)
 };

@@ -36,9 +36,6 @@ hvx_status get_encoder() {
     return g_encode ? HVX_SUCCESS : HVX_ERROR_DEVICE;
 }
 
-hvx_status encode_u8_map_at(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
-                            uint32_t h, uint32_t box_w, uint32_t box_h);
-
 // 2-D U8 tensor map of an image with a (box_w x box_h) box; out-of-image
 // elements of a box read as 0.
 hvx_status encode_u8_map(CUtensorMap* map, const Image* im, uint32_t box_w, uint32_t box_h) {
@@ -46,11 +43,13 @@ hvx_status encode_u8_map(CUtensorMap* map, const Image* im, uint32_t box_w, uint
         std::memset(map, 0, sizeof(*map));
         return HVX_SUCCESS;
     }
-    return encode_u8_map_at(map, im->dev, im->pitch, im->w, im->h, box_w, box_h);
+    return encode_map_raw(map, im->dev, im->pitch, im->w, im->h, box_w, box_h, 1);
 }
 
-hvx_status encode_u8_map_at(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
-                            uint32_t h, uint32_t box_w, uint32_t box_h) {
+}  // namespace
+
+hvx_status encode_map_raw(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
+                          uint32_t h, uint32_t box_w, uint32_t box_h, int elem_bytes) {
     hvx_status st = get_encoder();
     if (st != HVX_SUCCESS) return st;
     if (((uintptr_t)ptr & 15) || (pitch & 15)) return HVX_ERROR_INVALID_PARAMETERS;
@@ -59,11 +58,16 @@ hvx_status encode_u8_map_at(CUtensorMap* map, const void* ptr, uint64_t pitch, u
     cuuint64_t strides[1] = {pitch};
     cuuint32_t box[2] = {box_w, box_h};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, dev, dims, strides, box, estr,
+    CUresult r = g_encode(map,
+                          elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16
+                                          : CU_TENSOR_MAP_DATA_TYPE_UINT8,
+                          2, dev, dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? HVX_SUCCESS : HVX_ERROR_DEVICE;
 }
+
+namespace {
 
 void set_rect(int32_t* d, const Rect& r) {
     d[0] = r.x0;
@@ -834,7 +838,7 @@ struct BatchEntry {
     uint64_t last_use = 0;
     int grid = 0;  // persistent CTAs chosen by the autotuner
     // generated-kernel batches: one direct launch over every image's tiles
-    JitKernel* jk = nullptr;
+    JitBatch jit;
     int n = 0, total_tiles = 0;
     bool harris = false;  // BORDER_UNDEFINED corner batch: one direct launch
     bool tomasi = false;  // ... of the Shi-Tomasi kernel
@@ -1156,20 +1160,19 @@ hvx_status build_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int
 // Batch of graphs whose plans are one group running the same generated
 // kernel: the images' launch parameters and tile prefix sums in one device
 // block.
-hvx_status build_jit_batch_entry(Graph* const* gs, int n, JitKernel* jk, BatchEntry& out) {
-    int tw = 0, th = 0;
-    jit_tile(jk, &tw, &th);
+hvx_status build_jit_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEntry& out) {
+    std::vector<const JitLaunch*> js(n);
+    for (int i = 0; i < n; ++i) js[i] = &gs[i]->plan.groups[0].jit;
+    std::vector<HvxJitParams> ps(n);
+    std::vector<int> tiles(n);
+    hvx_status st = jit_batch_params(js.data(), n, ctx->num_sms, ps.data(), tiles.data(), &out.jit);
+    if (st != HVX_SUCCESS) return st;
     const size_t tiles_off = (size_t)n * sizeof(HvxJitParams);
     const size_t total = tiles_off + (size_t)(n + 1) * sizeof(int);
     std::vector<uint8_t> host(total);
     std::vector<int> tile_start(n + 1, 0);
-    for (int i = 0; i < n; ++i) {
-        const Group& G = gs[i]->plan.groups[0];
-        std::memcpy(host.data() + (size_t)i * sizeof(HvxJitParams), &G.jit.p, sizeof(HvxJitParams));
-        const long long t = (long long)tile_start[i] + (long long)G.jit.gx * G.jit.gy;
-        if (t > (1ll << 30)) return HVX_ERROR_NOT_SUPPORTED;
-        tile_start[i + 1] = (int)t;
-    }
+    for (int i = 0; i < n; ++i) tile_start[i + 1] = tile_start[i] + tiles[i];
+    std::memcpy(host.data(), ps.data(), tiles_off);
     std::memcpy(host.data() + tiles_off, tile_start.data(), (n + 1) * sizeof(int));
     void* dmem = nullptr;
     cudaError_t e = cudaMalloc(&dmem, total);
@@ -1186,9 +1189,6 @@ hvx_status build_jit_batch_entry(Graph* const* gs, int n, JitKernel* jk, BatchEn
     out.plan_ids.resize(n);
     for (int i = 0; i < n; ++i) out.plan_ids[i] = gs[i]->plan_id;
     out.dmem = dmem;
-    out.jk = jk;
-    out.n = n;
-    out.total_tiles = tile_start[n];
     return HVX_SUCCESS;
 }
 
@@ -1335,7 +1335,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             bc->entries.erase(oldest);
         }
         BatchEntry fresh;
-        hvx_status st = jit_same      ? build_jit_batch_entry(gs, n, jk, fresh)
+        hvx_status st = jit_same      ? build_jit_batch_entry(ctx, gs, n, fresh)
                         : harris_same ? build_harris_batch_entry(ctx, gs, n, fresh)
                                       : build_batch_entry(ctx, bc, gs, n, mode, s, fresh);
         if (st != HVX_SUCCESS) return st;
@@ -1343,7 +1343,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
         hit = &bc->entries.back();
     }
     hit->last_use = ++bc->tick;
-    if (hit->jk) {
+    if (hit->jit.k) {
         for (int i = 0; i < n; ++i)
             for (const ResultReset& rr : gs[i]->plan.groups[0].resets) {
                 cudaError_t e = cudaMemsetAsync(rr.p, rr.byte, rr.n, s);
@@ -1351,9 +1351,8 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             }
         const uint8_t* base = static_cast<const uint8_t*>(hit->dmem);
         return cuda_status(jit_launch_batch(
-            hit->jk, reinterpret_cast<const HvxJitParams*>(base),
-            reinterpret_cast<const int*>(base + (size_t)hit->n * sizeof(HvxJitParams)), hit->n,
-            hit->total_tiles, s));
+            hit->jit, reinterpret_cast<const HvxJitParams*>(base),
+            reinterpret_cast<const int*>(base + (size_t)n * sizeof(HvxJitParams)), s));
     }
     if (hit->harris) {
         const uint8_t* base = static_cast<const uint8_t*>(hit->dmem);
@@ -1367,11 +1366,6 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             hit->n, hit->total_tiles, hit->tomasi, hit->resp, s));
     }
     return cuda_status(cudaGraphLaunch(hit->exec, s));
-}
-
-hvx_status encode_u8_map_raw(CUtensorMap* map, const void* ptr, uint64_t pitch, uint32_t w,
-                             uint32_t h, uint32_t box_w, uint32_t box_h) {
-    return encode_u8_map_at(map, ptr, pitch, w, h, box_w, box_h);
 }
 
 }  // namespace hvx
