@@ -1649,6 +1649,18 @@ int set_tiles(const JitKernel& k, HvxJitParams& p, unsigned* gx, unsigned* gy) {
     return p.rows ? strip_smem_bytes(k.strip, p.rows) : k.smem_bytes;
 }
 
+// CTAs of an image with global operators: its share (by tiles) of the CTAs that
+// are resident at a time, so that each commits one partial result.
+int reduction_ctas(const JitKernel& k, const HvxJitParams& p, long long tiles, long long all,
+                   int num_sms) {
+    int per = 5;
+    if (k.fn && driver().occupancy(&per, k.fn, STRIP_THREADS,
+                                   (size_t)strip_smem_bytes(k.strip, p.rows)) != CUDA_SUCCESS)
+        per = 5;
+    const long long share = ((long long)std::max(per, 1) * num_sms * tiles + all - 1) / all;
+    return (int)std::max(1ll, std::min({tiles, share, (long long)STRIP_MAX_CTAS}));
+}
+
 // Tensor maps of the inputs that the launch's form stages by TMA.
 bool set_maps(const JitKernel& k, HvxJitParams& p) {
     static_assert(sizeof(HvxTensorMap) == sizeof(CUtensorMap), "tensor map blob");
@@ -1772,6 +1784,13 @@ JitKernel* find_kernel(const GenericDesc& d, const std::vector<std::string>& use
             slot->is_in[b] = em.ext_in[b] >= 0;
         }
         compile(*slot);
+        if (!slot->compiled && slot->strips) {  // the tile form instead
+            if (std::getenv("HVX_CODEGEN_VERBOSE"))
+                std::fprintf(stderr, "hvx: strip form does not compile: %s\n", slot->log.c_str());
+            slot->strips = false;
+            slot->source = em.o.str();
+            compile(*slot);
+        }
     }
     (*by_shape)[shape] = slot.get();
     return slot.get();
@@ -1819,6 +1838,10 @@ bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code
     const int rows = k->strips ? strip_rows(*k, &d.W, &d.H, 1, num_sms) : 0;
     p.rows = rows;
     j.smem = set_tiles(*k, p, &j.gx, &j.gy);
+    if (rows && k->strip.reduces) {
+        j.gx = (unsigned)(p.ctas = reduction_ctas(*k, p, j.gx * j.gy, j.gx * j.gy, num_sms));
+        j.gy = 1;
+    }
     if (load_module && !set_maps(*k, p)) {
         *why = "tensor map of a staged input";
         return false;
@@ -1882,13 +1905,22 @@ hvx_status jit_batch_params(const JitLaunch* const* js, int n, int num_sms, HvxJ
         total += tiles[i];
         if (!set_maps(k, p)) return HVX_ERROR_DEVICE;
     }
+    if (rows > 0 && k.strip.reduces) {  // blocks are CTAs of an image
+        const long long all = total;
+        total = 0;
+        for (int i = 0; i < n; ++i) {
+            out[i].ctas = reduction_ctas(k, out[i], tiles[i], all, num_sms);
+            tiles[i] = out[i].ctas;
+            total += tiles[i];
+        }
+    }
     if (total > (1ll << 30)) return HVX_ERROR_NOT_SUPPORTED;
     b->k = js[0]->k;
     b->n = n;
     b->rows = rows;
     b->gx = (unsigned)total;
     b->gy = b->gz = 1;
-    bool same = rows > 0 && n <= 65535;
+    bool same = rows > 0 && n <= 65535 && !k.strip.reduces;
     for (int i = 1; i < n; ++i) same = same && W[i] == W[0] && H[i] == H[0];
     b->uniform = same;
     if (same) {

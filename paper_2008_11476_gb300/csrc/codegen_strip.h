@@ -23,6 +23,7 @@ struct StripBox {
 struct StripPlan {
     int unroll = 0;  // rows per thread are a multiple of this
     std::vector<StripBox> boxes;
+    bool reduces = false;  // has global operators: p.ctas CTAs per image over its tiles
 };
 
 // Bytes of shared memory of a strip tile with `rows` rows per thread: the

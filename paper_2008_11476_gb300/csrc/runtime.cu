@@ -530,6 +530,9 @@ hvx_status build_eqhist(Plan& P, Group& G) {
     q.out = static_cast<uint8_t*>(op.out->dev);
     q.out_pitch = op.out->pitch;
     q.hist = static_cast<uint32_t*>(op.node->d_aux);
+    q.done = q.hist ? q.hist + 256 : nullptr;
+    q.lut = q.hist ? reinterpret_cast<uint8_t*>(q.hist + 260) : nullptr;
+    q.num_sms = op.out->ctx->num_sms > 0 ? op.out->ctx->num_sms : 152;
     set_rect(q.valid, op.in[0]->valid);
     if (op.out->ctx->plan_only) return HVX_SUCCESS;
     return q.in && q.out && q.hist ? HVX_SUCCESS : HVX_ERROR_INVALID_GRAPH;
@@ -695,7 +698,8 @@ hvx_status alloc_results(Plan& P, Context* ctx) {
     for (int i : P.order) {
         Op& op = P.ops[i];
         if (op_is_global(op.kind)) {
-            const uint64_t n = global_result_bytes(op.kind, op.node->p.hist_bins);
+            const uint64_t res = global_result_bytes(op.kind, op.node->p.hist_bins);
+            const uint64_t n = global_block_bytes(op.kind, op.node->p.hist_bins);
             if (op.out->dev && op.out->bytes != n) {
                 ctx->pool.free(op.out->dev);
                 op.out->dev = nullptr;
@@ -705,14 +709,16 @@ hvx_status alloc_results(Plan& P, Context* ctx) {
                 if (st != HVX_SUCCESS) return st;
                 op.out->owns_mem = true;
                 op.out->bytes = n;
-                cudaMemset(op.out->dev, global_result_fill(op.kind), n);
+                cudaMemset(op.out->dev, 0, n);
+                cudaMemset(op.out->dev, global_result_fill(op.kind), res);
             }
         }
         if (op.kind == OP_EQHIST && !op.node->d_aux) {
-            if (cudaMalloc(&op.node->d_aux, 256 * sizeof(uint32_t)) != cudaSuccess) {
+            if (cudaMalloc(&op.node->d_aux, EQHIST_BYTES) != cudaSuccess) {
                 cudaGetLastError();
                 return HVX_ERROR_NO_MEMORY;
             }
+            cudaMemset(op.node->d_aux, 0, EQHIST_BYTES);
         }
     }
     return HVX_SUCCESS;
@@ -747,9 +753,8 @@ hvx_status prepare_launches(Graph* g) {
         for (int i : G.ops) {
             const Op& op = P.ops[i];
             if (op_is_global(op.kind) && op.out->dev)
-                G.resets.push_back({op.out->dev, global_result_fill(op.kind), op.out->bytes});
-            if (op.kind == OP_EQHIST && op.node->d_aux)
-                G.resets.push_back({op.node->d_aux, 0, 256 * sizeof(uint32_t)});
+                G.resets.push_back({op.out->dev, global_result_fill(op.kind),
+                                    global_result_bytes(op.kind, op.node->p.hist_bins)});
         }
         if (G.ops.size() == 1 && first.kind == OP_EQHIST) {
             G.kernel = GK_EQHIST;
@@ -790,6 +795,8 @@ hvx_status prepare_launches(Graph* g) {
                 G.jit_on = jit_prepare(G.gdesc, G.user_code, !ctx->plan_only, ctx->device, &G.jit,
                                        &why);
                 G.jit.p.err = ctx->d_error;
+                // the strip form's last CTA writes the whole result
+                if (G.jit_on && G.jit.p.rows > 0) G.resets.clear();
                 if (!G.jit_on && getenv("HVX_CODEGEN_VERBOSE"))
                     fprintf(stderr, "hvx: no generated kernel for a group: %s\n", why.c_str());
                 if (!G.jit_on && (must_gen || user))

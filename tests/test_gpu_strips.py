@@ -126,3 +126,45 @@ def test_strip_and_tile_forms_agree(ctx, name, monkeypatch):
         H.hvxProcessGraph(g)
         got.append(PG.download(res[0][1]))
     np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (130, 40), (1031, 517)])
+@pytest.mark.parametrize("border", [H.HVX_BORDER_REPLICATE, H.HVX_BORDER_UNDEFINED])
+def test_global_operators_of_strips(ctx, w, h, border):
+    """MeanStdDev, MinMaxLoc and Histogram of images computed in the group (a
+    Gaussian, and its S16 difference from the input), run twice: the scratch of
+    the partial results is left clean.  Saturated areas, so that extrema are
+    taken by many pixels."""
+    img = synth.rects_noise(w, h, seed=h, sigma=40.0)
+    src = PG.upload(ctx, img, H.HVX_DF_U8)
+    g = H.hvxCreateGraph(ctx)
+    b, d = H.hvxCreateVirtualImage(g), H.hvxCreateVirtualImage(g, 0, 0, H.HVX_DF_S16)
+    H.hvxSetNodeBorder(H.hvxGaussian3x3Node(g, src, b), border, 0)
+    H.hvxSubtractNode(g, src, b, H.HVX_POLICY_SATURATE, d)
+    nodes = [H.hvxMeanStdDevNode(g, d), H.hvxMinMaxLocNode(g, b), H.hvxHistogramNode(g, b, 7, 20, 200),
+             H.hvxMinMaxLocNode(g, d)]
+    verified(g, H.HVX_CODEGEN_REQUIRE)
+    assert "hvx_generated_strips" in H.hvxGetGraphKernelSource(g, 0)
+    ob = O.BORDER_REPLICATE if border == H.HVX_BORDER_REPLICATE else O.BORDER_UNDEFINED
+    blur = O.gaussian3x3(img, ob)
+    x0, y0, x1, y1 = blur.rect
+    part = blur.data[y0:y1, x0:x1]
+    diff = img[y0:y1, x0:x1].astype(int) - part
+    for _ in range(2):
+        H.hvxProcessGraph(g)
+        m = H.hvxGetNodeResult(nodes[0], H.HvxMeanStdDev())
+        assert (m.sum, m.sum_squares, m.count) == (diff.sum(), (diff * diff).sum(), diff.size)
+        hist = H.hvxGetNodeResult(nodes[2], np.zeros(7, np.uint32))
+        v = part.astype(int)
+        want = np.bincount(((v - 20) * 7 // 200)[(v >= 20) & (v < 220)], minlength=7)
+        np.testing.assert_array_equal(hist, want)
+        for node, a in ((nodes[1], part.astype(int)), (nodes[3], diff)):
+            r = H.hvxGetNodeResult(node, H.HvxMinMaxLoc())
+            if a.size == 0:
+                assert (r.min_count, r.max_count, r.min_x) == (0, 0, -1)
+                continue
+            assert (r.min, r.max) == (a.min(), a.max())
+            assert (r.min_count, r.max_count) == ((a == a.min()).sum(), (a == a.max()).sum())
+            for at, (x, y) in ((a.argmin(), (r.min_x, r.min_y)), (a.argmax(), (r.max_x, r.max_y))):
+                assert (x, y) == (x0 + at % a.shape[1], y0 + at // a.shape[1])
+    H.hvxReleaseGraph(g)
