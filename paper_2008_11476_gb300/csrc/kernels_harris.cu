@@ -29,6 +29,7 @@
 // kernels below then evaluate tomasi_response_f32 on the window sums, the
 // binary32 function the point operator computes, and threshold its value.
 #include <atomic>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "launchers.h"
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(HARRIS_THREADS, 3)
 // Every thread runs all R rows (rows below the image read box rows the TMA
 // filled with 0 and are not stored), so the shuffles always see full warps.
 constexpr int FTW = 112, FTHREADS = 128;
-constexpr int FROWS_MIN = 8, FROWS_MAX = 24;  // boxes up to 144 x 198 bytes
+constexpr int FROWS_MIN = 3, FROWS_MAX = 24;  // boxes up to 144 x 198 bytes
 constexpr int FLW = FTW + 32;                 // box columns x0 - 16 .. x0 + 127
 constexpr int FLH_MAX = 8 * FROWS_MAX + 6;    // box rows y0 - 3 .. y0 + 8R + 2
 constexpr int RING = 5;        // gradient rows of the vertical window
@@ -530,14 +531,88 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
+// EDGE tiles under a border mode.  The Sobel's border mode on the box cells
+// of the one-pixel ring around the image (gradients further out are not used).
+__device__ void fill_ring(const HarrisParams& p, FastSmem& sm, int x0, int y0) {
+    if (p.border_s == HVX_BORDER_UNDEFINED) return;
+    const int W = p.W, H = p.H, bx = x0 - 16, by = y0 - 3, rows = 8 * p.rows + 6;
+    const bool cst = p.border_s == HVX_BORDER_CONSTANT;
+    auto set = [&](int x, int y) {
+        sm.in[y - by][x - bx] =
+            cst ? (uint8_t)p.cval_s : sm.in[clampi(y, 0, H - 1) - by][clampi(x, 0, W - 1) - bx];
+    };
+    const int c0 = max(bx, -1), c1 = min(bx + FLW - 1, W);
+    for (int x = c0 + (int)threadIdx.x; x <= c1; x += FTHREADS) {
+        if (by <= -1) set(x, -1);
+        if (H < by + rows) set(x, H);
+    }
+    for (int y = max(by, 0) + (int)threadIdx.x; y <= min(by + rows, H) - 1; y += FTHREADS) {
+        if (bx <= -1) set(-1, y);
+        if (W < bx + FLW) set(W, y);
+    }
+}
+
+// EDGE tiles: gradient row y (inside the image) of the strip at xs: zero
+// outside the gradients' valid rectangle, and columns outside the image as the
+// window sums read their products: the nearest column's (REPLICATE; it may
+// belong to the neighbouring strip) or zero (CONSTANT 0; UNDEFINED sums never
+// use them).  Every lane of the warp takes part.
+__device__ __forceinline__ void edge_grad(const HarrisParams& p, uint32_t* G, int xs, int y) {
+    const int W = p.W;
+    const bool rep = p.border_b == HVX_BORDER_REPLICATE;
+    const bool yok = y >= p.pvalid[1] && y < p.pvalid[3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int x = xs + 2 * j;
+        const uint32_t keep = (yok && x >= p.pvalid[0] && x < p.pvalid[2] ? 0xFFFFu : 0u) |
+                              (yok && x + 1 >= p.pvalid[0] && x + 1 < p.pvalid[2] ? 0xFFFF0000u : 0u);
+        G[j] = (G[j] & keep) | (0x04000400u & ~keep);
+        G[4 + j] = (G[4 + j] & keep) | (0x04000400u & ~keep);
+    }
+    if (!rep) return;  // (uniform)
+    // columns past W - 1 inside this strip
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t& g = G[4 * k + j];
+            const int x = xs + 2 * j;
+            if (x > W - 1 && j > 0) g = __byte_perm(G[4 * k + j - 1], 0u, 0x3232);
+            else if (x + 1 > W - 1) g = __byte_perm(g, 0u, 0x1010);
+        }
+    // strips wholly outside the image: the neighbour's nearest column
+    const uint32_t lx = __shfl_up_sync(0xffffffffu, G[3], 1), ly = __shfl_up_sync(0xffffffffu, G[7], 1);
+    const uint32_t rx = __shfl_down_sync(0xffffffffu, G[0], 1), ry = __shfl_down_sync(0xffffffffu, G[4], 1);
+    if (xs >= W || xs < 0) {
+        const uint32_t vx = xs < 0 ? __byte_perm(rx, 0u, 0x1010) : __byte_perm(lx, 0u, 0x3232);
+        const uint32_t vy = xs < 0 ? __byte_perm(ry, 0u, 0x1010) : __byte_perm(ly, 0u, 0x3232);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            G[j] = vx;
+            G[4 + j] = vy;
+        }
+    }
+}
+
+// Whether a tile's gradients and sums reach outside the image or the
+// gradients' valid rectangle under a border mode that reads them there.
+__device__ __forceinline__ bool edge_tile(const HarrisParams& p, int x0, int y0) {
+    if (p.border_s == HVX_BORDER_UNDEFINED && p.border_b == HVX_BORDER_UNDEFINED) return false;
+    return x0 - 3 < 0 || y0 - 3 < 0 || x0 + FTW + 3 > (int)p.W || y0 + 8 * p.rows + 3 > (int)p.H;
+}
+
 // One 112 x 8R output tile at (x0, y0) of the image that `tmap` / `p` describe.
 // RESP: the launch may export the response (p.resp); without it the row loop
-// holds only the mask path, which keeps the loop body small.
-template <bool TOMASI, bool RESP>
+// holds only the mask path, which keeps the loop body small.  EDGE: the tile
+// touches the image's border under a border mode that reads there.
+template <bool TOMASI, bool RESP, bool EDGE>
+__device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, FastSmem& sm, int x0,
+                                                      int y0);
+
+template <bool TOMASI, bool RESP, bool BORDER>
 __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const HarrisParams& p,
                                                  FastSmem& sm, int x0, int y0) {
     const int R = p.rows;
-    const int W = p.W, H = p.H;
     if (threadIdx.x == 0) {
         mbar_init(&sm.bar, 1);
         fence_barrier_init();
@@ -550,6 +625,20 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
     // every thread leaves together when the (bounded) wait ran out
     if (__syncthreads_or(!mbar_wait_bounded(&sm.bar, 0, p.err))) return;
 
+    if (BORDER && edge_tile(p, x0, y0)) {
+        fill_ring(p, sm, x0, y0);
+        __syncthreads();
+        harris_fast_rows_loop<TOMASI, RESP, true>(p, sm, x0, y0);
+    } else {
+        harris_fast_rows_loop<TOMASI, RESP, false>(p, sm, x0, y0);
+    }
+}
+
+template <bool TOMASI, bool RESP, bool EDGE>
+__device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, FastSmem& sm, int x0,
+                                                      int y0) {
+    const int R = p.rows;
+    const int W = p.W, H = p.H;
     const int q = threadIdx.x & 15, g = threadIdx.x >> 4;
     const int xs = x0 - 8 + 8 * q, yb = y0 + R * g;
     const bool producer = q >= 1 && q <= 14 && xs < W;
@@ -559,6 +648,7 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
     const bool full = xs >= p.valid[0] && xs + 8 <= p.valid[2] && yb >= p.valid[1] &&
                       yb + R <= p.valid[3];
     const int kn = (int)p.kn, kd = (int)p.kd;
+    const unsigned rcp = RESP && !TOMASI ? ratio_rcp(kd) : 0u;
     const HarrisDecide2 dk = harris_decide_consts(kn, kd, p.q_thr);
     const TomasiDecide2 tk = tomasi_decide_consts(p.thr_f);
     VSums V;
@@ -570,12 +660,30 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
     }
     // prologue: gradient rows yb - 2 .. yb + 1 (input rows yb - 3 .. yb + 2)
     uint32_t A[6], B[6], C[6], G[8];
-    load_pairs6(row, c, A);
-    load_pairs6(row + FLW, c, B);
+    const bool zero_rows = EDGE && p.border_b != HVX_BORDER_REPLICATE;
+    if (!EDGE) {
+        load_pairs6(row, c, A);
+        load_pairs6(row + FLW, c, B);
+    }
 #pragma unroll 1
     for (int r = 0; r < 4; ++r) {
-        load_pairs6(row + (r + 2) * FLW, c, C);
-        grad_row(A, B, C, G);
+        if (EDGE) {
+            // the gradient row of the nearest image row, or zero outside it
+            const int y = yb - 2 + r, yc = clampi(y, 0, H - 1);
+            const uint8_t* src = &sm.in[yc - 1 - (y0 - 3)][0];
+            load_pairs6(src, c, A);
+            load_pairs6(src + FLW, c, B);
+            load_pairs6(src + 2 * FLW, c, C);
+            grad_row(A, B, C, G);
+            edge_grad(p, G, xs, yc);
+            if (zero_rows && y != yc) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) G[k] = 0x04000400u;
+            }
+        } else {
+            load_pairs6(row + (r + 2) * FLW, c, C);
+            grad_row(A, B, C, G);
+        }
         ring[2 * r + 0] = make_uint4(G[0], G[1], G[2], G[3]);
         ring[2 * r + 1] = make_uint4(G[4], G[5], G[6], G[7]);
         add_products(G, V);
@@ -584,6 +692,10 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
             A[k] = B[k];
             B[k] = C[k];
         }
+    }
+    if (EDGE) {  // input rows yb + 1, yb + 2
+        load_pairs6(row + 4 * FLW, c, A);
+        load_pairs6(row + 5 * FLW, c, B);
     }
     uint8_t* mrow = p.mask ? p.mask + (size_t)yb * p.mask_pitch : nullptr;
     float* rrow = RESP && p.resp ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(p.resp) +
@@ -596,7 +708,17 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
         const int y = yb + i;
         // new gradient row y + 2 (input rows y + 1 .. y + 3) into ring slot (i + 4) mod 5
         load_pairs6(row + (i + 6) * FLW, c, Pn);
-        grad_row(Pa, Pb, Pn, G);
+        if (EDGE) {
+            uint32_t N[8];
+            grad_row(Pa, Pb, Pn, N);
+            edge_grad(p, N, xs, y + 2);
+            // rows below the image keep the last one's gradients, or zero
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                G[k] = y + 2 < H ? N[k] : zero_rows ? 0x04000400u : G[k];
+        } else {
+            grad_row(Pa, Pb, Pn, G);
+        }
         const int sn = (i + 4) % RING, so = i % RING;
         ring[2 * sn + 0] = make_uint4(G[0], G[1], G[2], G[3]);
         ring[2 * sn + 1] = make_uint4(G[4], G[5], G[6], G[7]);
@@ -699,7 +821,7 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
                     } else {  // the response is exported: exact q for both
                         const long long qv = harris_q32(ha[j], hb[j], hc[j], kn, kd);
                         hit = qv > p.q_thr;
-                        rv[j] = ok ? ratio_to_float(qv, p.kd) : 0.0f;
+                        rv[j] = ok ? ratio_to_float_rcp(qv, (unsigned)kd, rcp) : 0.0f;
                     }
                     mk[j] = ok ? (hit ? (uint32_t)p.tv : (uint32_t)p.fv) & 0xFFu : 0u;
                 }
@@ -741,14 +863,14 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
     }
 }
 
-template <bool TOMASI, bool RESP>
+template <bool TOMASI, bool RESP, bool BORDER>
 __global__ void __launch_bounds__(FTHREADS, 4)
     harris_fast_kernel(const __grid_constant__ CUtensorMap tmap, const HarrisParams p) {
     pdl_launch_dependents();  // launched by launch_pdl
     pdl_wait();
     extern __shared__ __align__(128) uint8_t smem_raw[];
     FastSmem& sm = *reinterpret_cast<FastSmem*>(smem_raw);
-    harris_fast_tile<TOMASI, RESP>(&tmap, p, sm, blockIdx.x * FTW, blockIdx.y * 8 * p.rows);
+    harris_fast_tile<TOMASI, RESP, BORDER>(&tmap, p, sm, blockIdx.x * FTW, blockIdx.y * 8 * p.rows);
 }
 
 // Several images in one launch (hvxProcessGraphBatch): block t is tile
@@ -756,11 +878,12 @@ __global__ void __launch_bounds__(FTHREADS, 4)
 // and parameters in global memory, all images with the same rows per thread
 // and the same response (Harris or Shi-Tomasi: TOMASI); RESP: some image
 // exports its response.
-template <bool TOMASI, bool RESP>
+template <bool TOMASI, bool RESP, bool BORDER>
 __global__ void __launch_bounds__(FTHREADS, 4)
     harris_fast_batch_kernel(const CUtensorMap* __restrict__ maps,
                              const HarrisParams* __restrict__ ps, const int* __restrict__ tile_start,
                              const int* __restrict__ tiles_x, int n) {
+    pdl_launch_dependents();  // launched by launch_pdl; the tables were there before
     extern __shared__ __align__(128) uint8_t smem_raw[];
     FastSmem& sm = *reinterpret_cast<FastSmem*>(smem_raw);
     const int t = blockIdx.x;
@@ -774,15 +897,17 @@ __global__ void __launch_bounds__(FTHREADS, 4)
     if (threadIdx.x < PW)
         reinterpret_cast<uint32_t*>(&sm.prm)[threadIdx.x] =
             __ldg(reinterpret_cast<const uint32_t*>(ps + i) + threadIdx.x);
+    pdl_wait();
     __syncthreads();
-    harris_fast_tile<TOMASI, RESP>(maps + i, sm.prm, sm, (local - ty * tx) * FTW,
+    harris_fast_tile<TOMASI, RESP, BORDER>(maps + i, sm.prm, sm, (local - ty * tx) * FTW,
                                    ty * 8 * sm.prm.rows);
 }
 
 }  // namespace
 
 bool harris_fast_path(const HarrisParams& p) {
-    return p.border_s == HVX_BORDER_UNDEFINED && p.border_b == HVX_BORDER_UNDEFINED && p.wr == 2 &&
+    // (a constant product other than 0 outside the image is no gradient's)
+    return (p.border_b != HVX_BORDER_CONSTANT || p.cval_b == 0) && p.wr == 2 &&
            p.rows >= FROWS_MIN && p.rows <= FROWS_MAX;
 }
 
@@ -844,46 +969,60 @@ cudaError_t set_fast_smem(K kernel, std::atomic<bool>& done) {
 }
 }  // namespace
 
-template <bool TOMASI, bool RESP>
+template <bool TOMASI, bool RESP, bool BORDER>
 cudaError_t launch_harris_batch_t(const CUtensorMap* maps, const HarrisParams* ps,
                                   const int* tile_start, const int* tiles_x, int n, int total,
                                   cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    cudaError_t e = set_fast_smem(harris_fast_batch_kernel<TOMASI, RESP>, attr);
+    cudaError_t e = set_fast_smem(harris_fast_batch_kernel<TOMASI, RESP, BORDER>, attr);
     if (e != cudaSuccess) return e;
-    harris_fast_batch_kernel<TOMASI, RESP><<<total, FTHREADS, (int)sizeof(FastSmem), s>>>(
-        maps, ps, tile_start, tiles_x, n);
-    return cudaGetLastError();
+    return launch_pdl(harris_fast_batch_kernel<TOMASI, RESP, BORDER>, dim3(total), dim3(FTHREADS),
+                      sizeof(FastSmem), s, maps, ps, tile_start, tiles_x, n);
 }
 
-template <bool TOMASI, bool RESP>
+template <bool TOMASI, bool RESP, bool BORDER>
 cudaError_t launch_harris_fast_t(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    cudaError_t e = set_fast_smem(harris_fast_kernel<TOMASI, RESP>, attr);
+    cudaError_t e = set_fast_smem(harris_fast_kernel<TOMASI, RESP, BORDER>, attr);
     if (e != cudaSuccess) return e;
     dim3 grid((p.W + FTW - 1) / FTW, (p.H + 8 * p.rows - 1) / (8 * p.rows));
-    return launch_pdl(harris_fast_kernel<TOMASI, RESP>, grid, dim3(FTHREADS), sizeof(FastSmem), s,
-                      map, p);
+    return launch_pdl(harris_fast_kernel<TOMASI, RESP, BORDER>, grid, dim3(FTHREADS),
+                      sizeof(FastSmem), s, map, p);
+}
+
+namespace {
+// f(TOMASI, RESP, BORDER) with the three as compile-time constants
+template <class F>
+cudaError_t by_variant(bool tomasi, bool resp, bool border, F f) {
+    using T = std::true_type;
+    using N = std::false_type;
+    if (tomasi)
+        return resp ? (border ? f(T{}, T{}, T{}) : f(T{}, T{}, N{}))
+                    : (border ? f(T{}, N{}, T{}) : f(T{}, N{}, N{}));
+    return resp ? (border ? f(N{}, T{}, T{}) : f(N{}, T{}, N{}))
+                : (border ? f(N{}, N{}, T{}) : f(N{}, N{}, N{}));
+}
+}  // namespace
+
+bool harris_borders(const HarrisParams& p) {
+    return p.border_s != HVX_BORDER_UNDEFINED || p.border_b != HVX_BORDER_UNDEFINED;
 }
 
 cudaError_t launch_harris_batch(const CUtensorMap* maps, const HarrisParams* ps,
                                 const int* tile_start, const int* tiles_x, int n, int total,
-                                bool tomasi, bool resp, cudaStream_t s) {
-    if (tomasi)
-        return resp ? launch_harris_batch_t<true, true>(maps, ps, tile_start, tiles_x, n, total, s)
-                    : launch_harris_batch_t<true, false>(maps, ps, tile_start, tiles_x, n, total, s);
-    return resp ? launch_harris_batch_t<false, true>(maps, ps, tile_start, tiles_x, n, total, s)
-                : launch_harris_batch_t<false, false>(maps, ps, tile_start, tiles_x, n, total, s);
+                                bool tomasi, bool resp, bool borders, cudaStream_t s) {
+    return by_variant(tomasi, resp, borders, [&](auto t, auto r, auto b) {
+        return launch_harris_batch_t<t.value, r.value, b.value>(maps, ps, tile_start, tiles_x, n,
+                                                                total, s);
+    });
 }
 
 cudaError_t launch_harris(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s) {
-    if (harris_fast_path(p)) {
-        if (p.tomasi)
-            return p.resp ? launch_harris_fast_t<true, true>(map, p, s)
-                          : launch_harris_fast_t<true, false>(map, p, s);
-        return p.resp ? launch_harris_fast_t<false, true>(map, p, s)
-                      : launch_harris_fast_t<false, false>(map, p, s);
-    }
+    if (harris_fast_path(p))
+        return by_variant(p.tomasi != 0, p.resp != nullptr, harris_borders(p),
+                          [&](auto t, auto r, auto b) {
+                              return launch_harris_fast_t<t.value, r.value, b.value>(map, p, s);
+                          });
     static bool attr_set = false;
     const int smem = (int)sizeof(HarrisSmem);
     if (!attr_set) {

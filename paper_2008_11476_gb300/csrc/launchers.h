@@ -54,18 +54,19 @@ cudaError_t launch_binom5(const CUtensorMap& map, const EdgeParams& p, cudaStrea
 cudaError_t launch_binom5_batch(const EdgeBatchDesc& d, int grid, int rows, cudaStream_t s);
 int binom5_batch_blocks_per_sm();
 
-// Harris: the UNDEFINED-border fast kernel or the general one; the tensor map
+// Harris: the strip kernel (harris_fast_path) or the general one; the tensor map
 // of the group's input must use the box harris_box() gives.
 bool harris_fast_path(const HarrisParams& p);
 int harris_fast_rows(int W, int H, int num_sms);
 void harris_box(const HarrisParams& p, int* w, int* h);
 cudaError_t launch_harris(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s);
-// BORDER_UNDEFINED Harris over n images in one launch (every image's rows
+// harris_fast_path groups over n images in one launch (every image's rows
 // equal; tensor maps boxed for them); total = tile_start[n]; resp: some
-// image exports its response
+// image exports its response; borders: some image has harris_borders()
+bool harris_borders(const HarrisParams& p);
 cudaError_t launch_harris_batch(const CUtensorMap* maps, const HarrisParams* ps,
                                 const int* tile_start, const int* tiles_x, int n, int total,
-                                bool tomasi, bool resp, cudaStream_t s);
+                                bool tomasi, bool resp, bool borders, cudaStream_t s);
 int harris_fast_tile_w();
 int harris_batch_rows(const int* W, const int* H, int n, int num_sms);
 cudaError_t launch_generic(const GenericDesc& d, cudaStream_t s);

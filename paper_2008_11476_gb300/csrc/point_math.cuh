@@ -88,39 +88,45 @@ __device__ __forceinline__ long long harris_q(int a, int b, int c, long long kn,
     return kd * det - kn * tr * tr;
 }
 
-// Binary32 value nearest to m / d (ties to even), m < 2^62, 1 <= d <= 1000:
-// a candidate from two correctly rounded steps (m to binary32, then the
-// division) is within about one unit in the last place; it is then moved to
-// the correctly rounded value by exact integer comparisons against the
-// midpoints to its neighbours.
-__device__ __forceinline__ float ratio_to_float(long long q, long long d) {
+// Binary32 value nearest to q / d (ties to even), |q| < 2^62, 1 <= d <= 1000.
+// Schoolbook division in 32-bit steps: with |q| shifted up so that its top bit
+// is bit 63, the upper 48 bits are divided by d in two digits (32 and 16 bits,
+// each by a multiplication with rcp = floor((2^32 - 1) / d), whose quotient is
+// at most one too small).  The 38 or more quotient bits, with a set last bit
+// when anything below them is left, round to 24 bits as the exact value does,
+// and the shift is undone by an exact power of two.  About 45 instructions
+// (with 128-bit comparisons against the neighbours' midpoints it took some 200:
+// the Harris response of a 1020x1020 frame 23.9 us).
+__device__ __forceinline__ unsigned int ratio_rcp(int d) { return 0xFFFFFFFFu / (unsigned int)d; }
+
+__device__ __forceinline__ float ratio_to_float_rcp(long long q, unsigned int d, unsigned int rcp) {
     if (q == 0) return 0.0f;
-    bool neg = q < 0;
-    unsigned long long m = neg ? (unsigned long long)(-q) : (unsigned long long)q;
-    float c = __fdiv_rn(__ull2float_rn(m), (float)d);
-    for (int it = 0; it < 4; ++it) {
-        int e;
-        float fr = frexpf(c, &e);                      // c = fr * 2^e, fr in [1/2, 1)
-        unsigned int M = (unsigned int)ldexpf(fr, 24); // c = M * 2^(e - 24)
-        int sh = 2 - (e - 24);                         // compare m * 2^sh with (4M +- k) d
-        unsigned __int128 L = m;
-        unsigned __int128 Hi = (unsigned __int128)(4ull * M + 2ull) * (unsigned long long)d;
-        unsigned __int128 Lo =
-            (unsigned __int128)(4ull * M - (M == (1u << 23) ? 1ull : 2ull)) * (unsigned long long)d;
-        if (sh >= 0) {
-            L <<= sh;
-        } else {
-            Hi <<= -sh;
-            Lo <<= -sh;
-        }
-        if (L > Hi || (L == Hi && (M & 1u)))
-            c = nextafterf(c, 3.0e38f);
-        else if (L < Lo || (L == Lo && (M & 1u)))
-            c = nextafterf(c, 0.0f);
-        else
-            break;
+    const unsigned long long m = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
+    const int lz = __clzll((long long)m);
+    const unsigned long long M = m << lz;
+    const unsigned int hi = (unsigned int)(M >> 32), lo = (unsigned int)M;
+    unsigned int q1 = __umulhi(hi, rcp), r = hi - q1 * d;
+    if (r >= d) {
+        ++q1;
+        r -= d;
     }
-    return neg ? -c : c;
+    const unsigned int n = (r << 16) | (lo >> 16);  // < 1000 * 2^16
+    unsigned int q2 = __umulhi(n, rcp);
+    r = n - q2 * d;
+    if (r >= d) {
+        ++q2;
+        r -= d;
+    }
+    const unsigned int sticky = (r | (lo & 0xFFFFu)) ? 1u : 0u;
+    const float f =
+        __ull2float_rn(((unsigned long long)q1 << 16) | (unsigned long long)(q2 | sticky));
+    // q1 2^16 + q2 = floor(M / 2^16 / d) = floor(m 2^(lz - 16) / d)
+    const float v = f * __int_as_float((127 + 16 - lz) << 23);
+    return q < 0 ? -v : v;
+}
+
+__device__ __forceinline__ float ratio_to_float(long long q, long long d) {
+    return ratio_to_float_rcp(q, (unsigned int)d, ratio_rcp((int)d));
 }
 
 // ---------------------------------------------------------------------------

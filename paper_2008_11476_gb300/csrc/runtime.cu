@@ -847,9 +847,10 @@ struct BatchEntry {
     // generated-kernel batches: one direct launch over every image's tiles
     JitBatch jit;
     int n = 0, total_tiles = 0;
-    bool harris = false;  // BORDER_UNDEFINED corner batch: one direct launch
+    bool harris = false;  // corner batch: one direct launch
     bool tomasi = false;  // ... of the Shi-Tomasi kernel
     bool resp = false;    // ... where some image exports its response
+    bool borders = false;  // ... where some image has a border mode
     std::vector<int> rows;  // edge batch: rows per thread of each image's tiles
     std::vector<void*> more_dmem;  // edge batch split by size class: the other tables
 };
@@ -1199,7 +1200,7 @@ hvx_status build_jit_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEnt
     return HVX_SUCCESS;
 }
 
-// Batch of BORDER_UNDEFINED Harris graphs: one rows-per-thread for all of
+// Batch of corner graphs on the strip kernel: one rows-per-thread for all of
 // them, each input's tensor map boxed for it, then maps, parameters and tile
 // tables in one device block.
 hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEntry& out) {
@@ -1250,7 +1251,10 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
     out.harris = true;
     out.tomasi = gs[0]->plan.groups[0].harris.tomasi != 0;
     out.resp = false;
-    for (int i = 0; i < n; ++i) out.resp = out.resp || gs[i]->plan.groups[0].harris.resp != nullptr;
+    for (int i = 0; i < n; ++i) {
+        out.resp = out.resp || gs[i]->plan.groups[0].harris.resp != nullptr;
+        out.borders = out.borders || harris_borders(gs[i]->plan.groups[0].harris);
+    }
     out.n = n;
     out.total_tiles = tile_start[n];
     return HVX_SUCCESS;
@@ -1286,7 +1290,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
                    P.groups[0].jit_on && (!jk || P.groups[0].jit.k == jk);
         if (jit_same) jk = P.groups[0].jit.k;
     }
-    // one launch when every plan is a single BORDER_UNDEFINED corner group
+    // one launch when every plan is a single corner group on the strip kernel
     // with the same response (Harris or Shi-Tomasi)
     bool harris_same = !jit_same;
     for (int i = 0; i < n && harris_same; ++i) {
@@ -1370,7 +1374,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             reinterpret_cast<const CUtensorMap*>(base),
             reinterpret_cast<const HarrisParams*>(base + params_off),
             reinterpret_cast<const int*>(base + tiles_off), reinterpret_cast<const int*>(base + tx_off),
-            hit->n, hit->total_tiles, hit->tomasi, hit->resp, s));
+            hit->n, hit->total_tiles, hit->tomasi, hit->resp, hit->borders, s));
     }
     return cuda_status(cudaGraphLaunch(hit->exec, s));
 }
