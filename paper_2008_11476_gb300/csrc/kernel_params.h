@@ -228,7 +228,9 @@ struct HarrisParams {
     int32_t border_b, cval_b;  // how the window sums read the products
     int32_t wr;                // window radius (2 for 5x5)
     int32_t tv, fv;
-    int32_t rows;              // BORDER_UNDEFINED kernel: output rows per thread
+    int32_t rows;              // strip kernel: output rows per thread
+    int32_t lanes;             // strip kernel: strips per row of threads (16 or 32)
+    int32_t pad;
     int32_t tomasi;            // 1: Shi-Tomasi response instead of Harris's
     float thr_f;               // Shi-Tomasi: mask = (binary32 response > thr_f)
     int64_t kn, kd;

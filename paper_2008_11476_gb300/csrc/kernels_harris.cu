@@ -244,16 +244,18 @@ __global__ void __launch_bounds__(HARRIS_THREADS, 3)
     }
 }
 
-// ---- BORDER_UNDEFINED fast path ------------------------------------------------------
+// ---- strip kernel ------------------------------------------------------
 // When both the Sobel and the window sums leave their border UNDEFINED, no
 // valid output reads a gradient or product outside the image or outside its
-// valid region, so no border fix-up is needed anywhere.  One CTA (128
-// threads) computes a 112 x 8R output tile from one TMA box of 144 x (8R + 6)
-// input bytes.  Thread (q, g) owns the 8 columns xs = x0 - 8 + 8q .. xs + 7
-// (q = 0 .. 15) and R rows; strips 1 .. 14 produce the outputs, strips 0 and
-// 15 only provide the vertical sums of the halo columns to their neighbours.
-// R (8 .. 24) is chosen per image size at plan time so that the busiest SM
-// walks the fewest rows (harris_fast_rows); 4 CTAs share an SM.
+// valid region, so no border fix-up is needed anywhere (under other border
+// modes the tiles on the image's border fix their gradients, edge_grad).  One
+// CTA (128 threads) computes a 112 x 8R output tile from one TMA box of 144 x
+// (8R + 6) input bytes (or 240 x 4R from two boxes, see NL).  Thread (q, g)
+// owns the 8 columns xs = x0 - 8 + 8q .. xs + 7 (q = 0 .. NL - 1) and R rows;
+// strips 1 .. NL - 2 produce the outputs, the first and the last only provide
+// the vertical sums of the halo columns to their neighbours.  R (3 .. 24) is
+// chosen per image size at plan time so that the busiest SM walks the fewest
+// rows (harris_fast_shape); 4 CTAs share an SM.
 // Each thread walks down its rows (three per loop trip, so the input windows
 // rotate by renaming):
 //   * each step forms one new gradient row (gx, gy at its 8 columns) in
@@ -275,17 +277,31 @@ __global__ void __launch_bounds__(HARRIS_THREADS, 3)
 //     the general kernel.
 // Every thread runs all R rows (rows below the image read box rows the TMA
 // filled with 0 and are not stored), so the shuffles always see full warps.
-constexpr int FTW = 112, FTHREADS = 128;
-constexpr int FROWS_MIN = 3, FROWS_MAX = 24;  // boxes up to 144 x 198 bytes
-constexpr int FLW = FTW + 32;                 // box columns x0 - 16 .. x0 + 127
-constexpr int FLH_MAX = 8 * FROWS_MAX + 6;    // box rows y0 - 3 .. y0 + 8R + 2
+constexpr int FTHREADS = 128;
+constexpr int FROWS_MIN = 3, FROWS_MAX = 24;
+constexpr int FLW = 144;       // box columns x0 - 16 .. x0 + 127
+// Strips per row of threads, NL: 16 (112 columns x 8R rows from one box of 8R
+// + 6 rows) or 32 (240 columns x 4R rows from two boxes of 4R + 6 rows, the
+// second 128 columns further right).  Two strips of each row only provide halo
+// sums: 12.5 % of the lanes at 16 strips, 6.25 % at 32.
+constexpr int FBOX_STEP = 128;
+__host__ __device__ constexpr int fast_tw(int nl) { return 8 * (nl - 2); }
+__host__ __device__ constexpr int fast_groups(int nl) { return FTHREADS / nl; }
+__host__ __device__ constexpr int fast_box_rows(int nl, int R) { return fast_groups(nl) * R + 6; }
+// Shared-memory row of the second box: a multiple of 8, so that its first byte
+// is 128-byte aligned, as a TMA destination has to be.
+__host__ __device__ constexpr int fast_box1_row(int R) { return (fast_box_rows(32, R) + 7) & ~7; }
+static_assert(8 * FLW % 128 == 0, "8 box rows keep the alignment");
+constexpr int FLH_MAX = fast_box1_row(FROWS_MAX) + fast_box_rows(32, FROWS_MAX);
+static_assert(FLH_MAX >= fast_box_rows(16, FROWS_MAX), "one box of 16 strips fits");
 constexpr int RING = 5;        // gradient rows of the vertical window
 constexpr int RSTRIDE = 11;    // 16-byte units per thread: 5 rows x 2 + 1 (odd: no conflicts)
-static_assert(FTHREADS == 16 * 8, "16 strips x 8 row groups");
-static_assert(FTW % 16 == 0, "TMA boxes start on 16-byte columns");
+static_assert(fast_tw(16) % 16 == 0 && fast_tw(32) % 16 == 0 && FBOX_STEP % 16 == 0,
+              "TMA boxes start on 16-byte columns");
 
 struct FastSmem {
-    alignas(128) uint8_t in[FLH_MAX][FLW];  // image (x0 - 16 + c, y0 - 3 + r)
+    // image (x0 - 16 + c, y0 - 3 + r); 32 strips: then the second box's rows
+    alignas(128) uint8_t in[FLH_MAX][FLW];
     alignas(16) uint4 ring[FTHREADS][RSTRIDE];
     alignas(8) uint64_t bar;
     HarrisParams prm;  // batch: this tile's image parameters
@@ -535,7 +551,7 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 // of the one-pixel ring around the image (gradients further out are not used).
 __device__ void fill_ring(const HarrisParams& p, FastSmem& sm, int x0, int y0) {
     if (p.border_s == HVX_BORDER_UNDEFINED) return;
-    const int W = p.W, H = p.H, bx = x0 - 16, by = y0 - 3, rows = 8 * p.rows + 6;
+    const int W = p.W, H = p.H, bx = x0 - 16, by = y0 - 3, rows = fast_box_rows(16, p.rows);
     const bool cst = p.border_s == HVX_BORDER_CONSTANT;
     auto set = [&](int x, int y) {
         sm.in[y - by][x - bx] =
@@ -598,18 +614,19 @@ __device__ __forceinline__ void edge_grad(const HarrisParams& p, uint32_t* G, in
 // gradients' valid rectangle under a border mode that reads them there.
 __device__ __forceinline__ bool edge_tile(const HarrisParams& p, int x0, int y0) {
     if (p.border_s == HVX_BORDER_UNDEFINED && p.border_b == HVX_BORDER_UNDEFINED) return false;
-    return x0 - 3 < 0 || y0 - 3 < 0 || x0 + FTW + 3 > (int)p.W || y0 + 8 * p.rows + 3 > (int)p.H;
+    return x0 - 3 < 0 || y0 - 3 < 0 || x0 + fast_tw(16) + 3 > (int)p.W ||
+           y0 + fast_groups(16) * p.rows + 3 > (int)p.H;
 }
 
-// One 112 x 8R output tile at (x0, y0) of the image that `tmap` / `p` describe.
+// One output tile at (x0, y0) of the image that `tmap` / `p` describe.
 // RESP: the launch may export the response (p.resp); without it the row loop
 // holds only the mask path, which keeps the loop body small.  EDGE: the tile
 // touches the image's border under a border mode that reads there.
-template <bool TOMASI, bool RESP, bool EDGE>
+template <bool TOMASI, bool RESP, bool EDGE, int NL>
 __device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, FastSmem& sm, int x0,
                                                       int y0);
 
-template <bool TOMASI, bool RESP, bool BORDER>
+template <bool TOMASI, bool RESP, bool BORDER, int NL>
 __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const HarrisParams& p,
                                                  FastSmem& sm, int x0, int y0) {
     const int R = p.rows;
@@ -619,31 +636,38 @@ __device__ __forceinline__ void harris_fast_tile(const CUtensorMap* tmap, const 
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        mbar_arrive_expect_tx(&sm.bar, (uint32_t)(FLW * (8 * R + 6)));
+        const int rows = fast_box_rows(NL, R);
+        mbar_arrive_expect_tx(&sm.bar, (uint32_t)(FLW * rows * (NL / 16)));
         tma_load_2d(&sm.in[0][0], tmap, &sm.bar, x0 - 16, y0 - 3);
+        if (NL == 32) tma_load_2d(&sm.in[fast_box1_row(R)][0], tmap, &sm.bar, x0 - 16 + FBOX_STEP, y0 - 3);
     }
     // every thread leaves together when the (bounded) wait ran out
     if (__syncthreads_or(!mbar_wait_bounded(&sm.bar, 0, p.err))) return;
 
-    if (BORDER && edge_tile(p, x0, y0)) {
-        fill_ring(p, sm, x0, y0);
-        __syncthreads();
-        harris_fast_rows_loop<TOMASI, RESP, true>(p, sm, x0, y0);
-    } else {
-        harris_fast_rows_loop<TOMASI, RESP, false>(p, sm, x0, y0);
+    if constexpr (BORDER) {
+        if (edge_tile(p, x0, y0)) {
+            fill_ring(p, sm, x0, y0);
+            __syncthreads();
+            harris_fast_rows_loop<TOMASI, RESP, true, NL>(p, sm, x0, y0);
+            return;
+        }
     }
+    harris_fast_rows_loop<TOMASI, RESP, false, NL>(p, sm, x0, y0);
 }
 
-template <bool TOMASI, bool RESP, bool EDGE>
+template <bool TOMASI, bool RESP, bool EDGE, int NL>
 __device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, FastSmem& sm, int x0,
                                                       int y0) {
+    static_assert(!EDGE || NL == 16, "border tiles have 16 strips");
     const int R = p.rows;
     const int W = p.W, H = p.H;
-    const int q = threadIdx.x & 15, g = threadIdx.x >> 4;
+    const int q = threadIdx.x & (NL - 1), g = threadIdx.x / NL;
     const int xs = x0 - 8 + 8 * q, yb = y0 + R * g;
-    const bool producer = q >= 1 && q <= 14 && xs < W;
-    const int c = 8 + 8 * q;
-    const uint8_t* row = &sm.in[R * g][0];  // input row yb - 3
+    const bool producer = q >= 1 && q <= NL - 2 && xs < W;
+    const bool second = NL == 32 && q >= 16;  // the strip's columns lie in the second box
+    const int c = 8 + 8 * q - (second ? FBOX_STEP : 0);
+    // input row yb - 3
+    const uint8_t* row = &sm.in[R * g + (second ? fast_box1_row(R) : 0)][0];
     uint4* ring = sm.ring[threadIdx.x];
     const bool full = xs >= p.valid[0] && xs + 8 <= p.valid[2] && yb >= p.valid[1] &&
                       yb + R <= p.valid[3];
@@ -852,6 +876,20 @@ __device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, Fas
         const uint32_t O[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
         sub_products(O, V);
     };
+    if (RESP || EDGE) {
+        // one row per trip: the step is long (exact responses, border fix-ups),
+        // and three copies of it stall on instruction fetch
+#pragma unroll 1
+        for (int i = 0; i < R; ++i) {
+            step(A, B, C, i);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                A[k] = B[k];
+                B[k] = C[k];
+            }
+        }
+        return;
+    }
     // three rows per trip: the input windows rotate by renaming
 #pragma unroll 1
     for (int i = 0; i < R; i += 3) {
@@ -863,14 +901,15 @@ __device__ __forceinline__ void harris_fast_rows_loop(const HarrisParams& p, Fas
     }
 }
 
-template <bool TOMASI, bool RESP, bool BORDER>
+template <bool TOMASI, bool RESP, bool BORDER, int NL>
 __global__ void __launch_bounds__(FTHREADS, 4)
     harris_fast_kernel(const __grid_constant__ CUtensorMap tmap, const HarrisParams p) {
     pdl_launch_dependents();  // launched by launch_pdl
     pdl_wait();
     extern __shared__ __align__(128) uint8_t smem_raw[];
     FastSmem& sm = *reinterpret_cast<FastSmem*>(smem_raw);
-    harris_fast_tile<TOMASI, RESP, BORDER>(&tmap, p, sm, blockIdx.x * FTW, blockIdx.y * 8 * p.rows);
+    harris_fast_tile<TOMASI, RESP, BORDER, NL>(&tmap, p, sm, blockIdx.x * fast_tw(NL),
+                                               blockIdx.y * fast_groups(NL) * p.rows);
 }
 
 // Several images in one launch (hvxProcessGraphBatch): block t is tile
@@ -878,7 +917,7 @@ __global__ void __launch_bounds__(FTHREADS, 4)
 // and parameters in global memory, all images with the same rows per thread
 // and the same response (Harris or Shi-Tomasi: TOMASI); RESP: some image
 // exports its response.
-template <bool TOMASI, bool RESP, bool BORDER>
+template <bool TOMASI, bool RESP, bool BORDER, int NL>
 __global__ void __launch_bounds__(FTHREADS, 4)
     harris_fast_batch_kernel(const CUtensorMap* __restrict__ maps,
                              const HarrisParams* __restrict__ ps, const int* __restrict__ tile_start,
@@ -899,11 +938,15 @@ __global__ void __launch_bounds__(FTHREADS, 4)
             __ldg(reinterpret_cast<const uint32_t*>(ps + i) + threadIdx.x);
     pdl_wait();
     __syncthreads();
-    harris_fast_tile<TOMASI, RESP, BORDER>(maps + i, sm.prm, sm, (local - ty * tx) * FTW,
-                                   ty * 8 * sm.prm.rows);
+    harris_fast_tile<TOMASI, RESP, BORDER, NL>(maps + i, sm.prm, sm, (local - ty * tx) * fast_tw(NL),
+                                               ty * fast_groups(NL) * sm.prm.rows);
 }
 
 }  // namespace
+
+bool harris_borders(const HarrisParams& p) {
+    return p.border_s != HVX_BORDER_UNDEFINED || p.border_b != HVX_BORDER_UNDEFINED;
+}
 
 bool harris_fast_path(const HarrisParams& p) {
     // (a constant product other than 0 outside the image is no gradient's)
@@ -911,51 +954,46 @@ bool harris_fast_path(const HarrisParams& p) {
            p.rows >= FROWS_MIN && p.rows <= FROWS_MAX;
 }
 
-// Rows per thread of the BORDER_UNDEFINED kernel for a W x H image on
-// `num_sms` SMs: the R that minimises (waves of 4 CTAs per SM) x (rows each
-// CTA walks, R plus the 4-row prologue).  Measured on 4096 x 2160: R = 17 (592
-// CTAs, one full wave) 41 us; R = 20 (518) and 23 (444 CTAs, SMs left with
-// fewer than 4) 49 us; R = 15 (666 CTAs, two waves) 54 us.
-int harris_fast_rows(int W, int H, int num_sms) {
-    const long tiles_x = (W + FTW - 1) / FTW;
+// Rows per thread R and strips per row NL of a launch over n images: those
+// that minimise (waves of 4 CTAs per SM) x (rows each CTA walks, R plus the
+// 4-row prologue), 16 strips where equal.  32 strips (mask alone, no border
+// tiles) suit widths that 240 divides better than 112 does: 16 x 1080p
+// Shi-Tomasi (8 tiles of 240 against 18 of 112 columns) 96.0 -> 89.8 us, 16 x
+// 4096x2160 Harris 293.0 -> 288.8 us.
+// Measured on one 4096 x 2160 frame (16 strips): R = 17 (592 CTAs, one full
+// wave) 41 us; R = 20 (518) and 23 (444 CTAs, SMs left with fewer than 4) 49
+// us; R = 15 (666 CTAs, two waves) 54 us.
+void harris_fast_shape(const int* W, const int* H, int n, bool wide_ok, int num_sms, int* rows,
+                       int* lanes) {
     const long slots = 4L * (num_sms > 0 ? num_sms : 1);
-    int best = FROWS_MAX;
+    *rows = FROWS_MAX;
+    *lanes = 16;
     long best_cost = -1;
-    for (int r = FROWS_MIN; r <= FROWS_MAX; ++r) {
-        const long tiles = tiles_x * ((H + 8 * r - 1) / (8 * r));
-        const long cost = (tiles + slots - 1) / slots * (r + 4);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = r;
+    for (int nl = 16; nl <= (wide_ok ? 32 : 16); nl += 16)
+        for (int r = FROWS_MIN; r <= FROWS_MAX; ++r) {
+            const int tw = fast_tw(nl), th = fast_groups(nl) * r;
+            long tiles = 0;
+            for (int i = 0; i < n; ++i)
+                tiles += (long)((W[i] + tw - 1) / tw) * ((H[i] + th - 1) / th);
+            const long cost = (tiles + slots - 1) / slots * (r + 4);
+            if (best_cost < 0 || cost < best_cost) {
+                best_cost = cost;
+                *rows = r;
+                *lanes = nl;
+            }
         }
-    }
-    return best;
+}
+
+bool harris_wide_ok(const HarrisParams& p) { return !p.resp && !harris_borders(p); }
+
+void harris_tile(const HarrisParams& p, int* w, int* h) {
+    *w = fast_tw(p.lanes);
+    *h = fast_groups(p.lanes) * p.rows;
 }
 
 void harris_box(const HarrisParams& p, int* w, int* h) {
     *w = harris_fast_path(p) ? FLW : HARRIS_LOAD_W;
-    *h = harris_fast_path(p) ? 8 * p.rows + 6 : HARRIS_TH + 6;
-}
-
-int harris_fast_tile_w() { return FTW; }
-
-// Rows per thread for a batch of images in one launch: the same wave model
-// as harris_fast_rows over the tiles of all images.
-int harris_batch_rows(const int* W, const int* H, int n, int num_sms) {
-    const long slots = 4L * (num_sms > 0 ? num_sms : 1);
-    int best = FROWS_MAX;
-    long best_cost = -1;
-    for (int r = FROWS_MIN; r <= FROWS_MAX; ++r) {
-        long tiles = 0;
-        for (int i = 0; i < n; ++i)
-            tiles += (long)((W[i] + FTW - 1) / FTW) * ((H[i] + 8 * r - 1) / (8 * r));
-        const long cost = (tiles + slots - 1) / slots * (r + 4);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = r;
-        }
-    }
-    return best;
+    *h = harris_fast_path(p) ? fast_box_rows(p.lanes, p.rows) : HARRIS_TH + 6;
 }
 
 namespace {
@@ -969,59 +1007,61 @@ cudaError_t set_fast_smem(K kernel, std::atomic<bool>& done) {
 }
 }  // namespace
 
-template <bool TOMASI, bool RESP, bool BORDER>
+template <bool TOMASI, bool RESP, bool BORDER, int NL>
 cudaError_t launch_harris_batch_t(const CUtensorMap* maps, const HarrisParams* ps,
                                   const int* tile_start, const int* tiles_x, int n, int total,
                                   cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    cudaError_t e = set_fast_smem(harris_fast_batch_kernel<TOMASI, RESP, BORDER>, attr);
+    cudaError_t e = set_fast_smem(harris_fast_batch_kernel<TOMASI, RESP, BORDER, NL>, attr);
     if (e != cudaSuccess) return e;
-    return launch_pdl(harris_fast_batch_kernel<TOMASI, RESP, BORDER>, dim3(total), dim3(FTHREADS),
-                      sizeof(FastSmem), s, maps, ps, tile_start, tiles_x, n);
+    return launch_pdl(harris_fast_batch_kernel<TOMASI, RESP, BORDER, NL>, dim3(total),
+                      dim3(FTHREADS), sizeof(FastSmem), s, maps, ps, tile_start, tiles_x, n);
 }
 
-template <bool TOMASI, bool RESP, bool BORDER>
+template <bool TOMASI, bool RESP, bool BORDER, int NL>
 cudaError_t launch_harris_fast_t(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s) {
     static std::atomic<bool> attr{false};
-    cudaError_t e = set_fast_smem(harris_fast_kernel<TOMASI, RESP, BORDER>, attr);
+    cudaError_t e = set_fast_smem(harris_fast_kernel<TOMASI, RESP, BORDER, NL>, attr);
     if (e != cudaSuccess) return e;
-    dim3 grid((p.W + FTW - 1) / FTW, (p.H + 8 * p.rows - 1) / (8 * p.rows));
-    return launch_pdl(harris_fast_kernel<TOMASI, RESP, BORDER>, grid, dim3(FTHREADS),
+    int tw = 0, th = 0;
+    harris_tile(p, &tw, &th);
+    dim3 grid((p.W + tw - 1) / tw, (p.H + th - 1) / th);
+    return launch_pdl(harris_fast_kernel<TOMASI, RESP, BORDER, NL>, grid, dim3(FTHREADS),
                       sizeof(FastSmem), s, map, p);
 }
 
 namespace {
-// f(TOMASI, RESP, BORDER) with the three as compile-time constants
+// f(TOMASI, RESP, BORDER, NL) as compile-time constants
 template <class F>
-cudaError_t by_variant(bool tomasi, bool resp, bool border, F f) {
+cudaError_t by_variant(bool tomasi, bool resp, bool border, int lanes, F f) {
     using T = std::true_type;
     using N = std::false_type;
+    using L16 = std::integral_constant<int, 16>;
+    using L32 = std::integral_constant<int, 32>;
+    if (lanes == 32) return tomasi ? f(T{}, N{}, N{}, L32{}) : f(N{}, N{}, N{}, L32{});
     if (tomasi)
-        return resp ? (border ? f(T{}, T{}, T{}) : f(T{}, T{}, N{}))
-                    : (border ? f(T{}, N{}, T{}) : f(T{}, N{}, N{}));
-    return resp ? (border ? f(N{}, T{}, T{}) : f(N{}, T{}, N{}))
-                : (border ? f(N{}, N{}, T{}) : f(N{}, N{}, N{}));
+        return resp ? (border ? f(T{}, T{}, T{}, L16{}) : f(T{}, T{}, N{}, L16{}))
+                    : (border ? f(T{}, N{}, T{}, L16{}) : f(T{}, N{}, N{}, L16{}));
+    return resp ? (border ? f(N{}, T{}, T{}, L16{}) : f(N{}, T{}, N{}, L16{}))
+                : (border ? f(N{}, N{}, T{}, L16{}) : f(N{}, N{}, N{}, L16{}));
 }
 }  // namespace
 
-bool harris_borders(const HarrisParams& p) {
-    return p.border_s != HVX_BORDER_UNDEFINED || p.border_b != HVX_BORDER_UNDEFINED;
-}
-
 cudaError_t launch_harris_batch(const CUtensorMap* maps, const HarrisParams* ps,
                                 const int* tile_start, const int* tiles_x, int n, int total,
-                                bool tomasi, bool resp, bool borders, cudaStream_t s) {
-    return by_variant(tomasi, resp, borders, [&](auto t, auto r, auto b) {
-        return launch_harris_batch_t<t.value, r.value, b.value>(maps, ps, tile_start, tiles_x, n,
-                                                                total, s);
+                                bool tomasi, bool resp, bool borders, int lanes, cudaStream_t s) {
+    return by_variant(tomasi, resp, borders, lanes, [&](auto t, auto r, auto b, auto l) {
+        return launch_harris_batch_t<t.value, r.value, b.value, l.value>(maps, ps, tile_start,
+                                                                         tiles_x, n, total, s);
     });
 }
 
 cudaError_t launch_harris(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s) {
     if (harris_fast_path(p))
-        return by_variant(p.tomasi != 0, p.resp != nullptr, harris_borders(p),
-                          [&](auto t, auto r, auto b) {
-                              return launch_harris_fast_t<t.value, r.value, b.value>(map, p, s);
+        return by_variant(p.tomasi != 0, p.resp != nullptr, harris_borders(p), p.lanes,
+                          [&](auto t, auto r, auto b, auto l) {
+                              return launch_harris_fast_t<t.value, r.value, b.value, l.value>(map,
+                                                                                              p, s);
                           });
     static bool attr_set = false;
     const int smem = (int)sizeof(HarrisSmem);

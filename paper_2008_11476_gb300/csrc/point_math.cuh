@@ -92,11 +92,12 @@ __device__ __forceinline__ long long harris_q(int a, int b, int c, long long kn,
 // Schoolbook division in 32-bit steps: with |q| shifted up so that its top bit
 // is bit 63, the upper 48 bits are divided by d in two digits (32 and 16 bits,
 // each by a multiplication with rcp = floor((2^32 - 1) / d), whose quotient is
-// at most one too small).  The 38 or more quotient bits, with a set last bit
-// when anything below them is left, round to 24 bits as the exact value does,
-// and the shift is undone by an exact power of two.  About 45 instructions
-// (with 128-bit comparisons against the neighbours' midpoints it took some 200:
-// the Harris response of a 1020x1020 frame 23.9 us).
+// at most one too small).  The top 32 of the 38 or more quotient bits, with a
+// set last bit when anything below them is left, round to 24 bits as the exact
+// value does, and the shifts are undone by an exact power of two.  About 45
+// instructions, none on 64-bit conversions (with 128-bit comparisons against
+// the neighbours' midpoints it took some 200: the Harris response of a
+// 1020x1020 frame 23.9 us, 14.0 with its strip kernel).
 __device__ __forceinline__ unsigned int ratio_rcp(int d) { return 0xFFFFFFFFu / (unsigned int)d; }
 
 __device__ __forceinline__ float ratio_to_float_rcp(long long q, unsigned int d, unsigned int rcp) {
@@ -117,11 +118,12 @@ __device__ __forceinline__ float ratio_to_float_rcp(long long q, unsigned int d,
         ++q2;
         r -= d;
     }
-    const unsigned int sticky = (r | (lo & 0xFFFFu)) ? 1u : 0u;
-    const float f =
-        __ull2float_rn(((unsigned long long)q1 << 16) | (unsigned long long)(q2 | sticky));
-    // q1 2^16 + q2 = floor(M / 2^16 / d) = floor(m 2^(lz - 16) / d)
-    const float v = f * __int_as_float((127 + 16 - lz) << 23);
+    // Q = q1 2^16 + q2 = floor(M / 2^16 / d), 2^21 < q1 (hi >= 2^31); its top 32
+    // bits, anything below them (at most 26 bits) in the last one
+    const int nz = __clz((int)q1);  // <= 10
+    const unsigned int rest = (q2 << (16 + nz)) | r | (lo & 0xFFFFu);
+    const unsigned int top = (q1 << nz) | (q2 >> (16 - nz)) | (rest ? 1u : 0u);
+    const float v = __uint2float_rn(top) * __int_as_float((127 + 32 - lz - nz) << 23);
     return q < 0 ? -v : v;
 }
 

@@ -78,3 +78,29 @@ def test_corner_kernel_borders(ctx, borders, tomasi):
         for got, ref in zip(outs, refs):
             for im, r in zip(got, ref):
                 np.testing.assert_array_equal(PG.download(im), r)
+
+
+@pytest.mark.parametrize("tomasi", [False, True])
+def test_wide_and_narrow_strip_rows_agree(ctx, tomasi):
+    """Mask alone (240-column tiles where they suit the width, 112 otherwise)
+    against the mask of the same graph exporting its response (112 columns
+    always); widths and heights around both tiles, single and batched."""
+    sizes = [(1920, 1080), (1913, 1079), (480, 4000), (479, 3997), (473, 4003), (2409, 611)]
+    graphs, masks, refs = [], [], []
+    for i, (w, h) in enumerate(sizes):
+        src = PG.upload(ctx, synth.rects_noise(w, h, seed=50 + i), H.HVX_DF_U8)
+        g, (mask,) = corner_graph(ctx, src, w, h, (U, 0, U, 0), tomasi, False)
+        g2, (want, _) = corner_graph(ctx, src, w, h, (U, 0, U, 0), tomasi, True)
+        H.hvxProcessGraph(g)
+        H.hvxProcessGraph(g2)
+        refs.append(PG.download(want))
+        np.testing.assert_array_equal(PG.download(mask), refs[-1], err_msg=f"{w}x{h}")
+        graphs.append(g)
+        masks.append(mask)
+    for m, r in zip(masks, refs):
+        stale = np.full_like(r, 7)
+        H.hvxCopyImage(m, stale.ctypes.data, stale.strides[0], H.HVX_WRITE)
+    H.hvxProcessGraphBatch(graphs)
+    H.hvxWaitBatch(ctx)
+    for m, r in zip(masks, refs):
+        np.testing.assert_array_equal(PG.download(m), r)

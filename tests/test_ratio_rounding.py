@@ -1,6 +1,6 @@
 """CPU replay of the kernels' binary32 rounding of q / d (the Harris response):
-the 32-bit digit division with a truncated reciprocal, the sticky bit and the
-final scaling, against the oracle's correctly rounded ratio, on random values
+the 32-bit digit division with a truncated reciprocal, the bits kept, the sticky
+bit and the final scaling, against the oracle's correctly rounded ratio, on random values
 of every magnitude, ties and near-ties, and every divisor the response takes."""
 import numpy as np
 import pytest
@@ -28,9 +28,13 @@ def ratio(q, d):
     assert 0 <= r < 2 * d and q2 < 1 << 16
     if r >= d:
         q2, r = q2 + 1, r - d
-    Q = (q1 << 16) | q2 | (1 if r or lo & 0xFFFF else 0)
-    # an integer to binary32, ties to even (numpy rounds 64-bit integers once)
-    f = np.float32(np.uint64(Q)) * np.float32(2.0 ** (16 - lz))
+    nz = 32 - q1.bit_length()
+    assert 0 <= nz <= 10
+    rest = ((q2 << (16 + nz)) & 0xFFFFFFFF) | r | (lo & 0xFFFF)
+    top = (q1 << nz) | (q2 >> (16 - nz)) | (1 if rest else 0)
+    assert 1 << 31 <= top < 1 << 32
+    # an integer to binary32, ties to even (numpy rounds integers once)
+    f = np.float32(np.uint32(top)) * np.float32(2.0 ** (32 - lz - nz))
     return -f if q < 0 else f
 
 
