@@ -41,6 +41,8 @@
 // The batch kernel runs the same tile code persistently over the tiles of
 // many images (one tensor map and parameter block per image) with two boxes
 // in flight per CTA.
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "launchers.h"
 
@@ -1001,15 +1003,27 @@ int edge_mode(const EdgeParams& p) {
     return M_PHASE;
 }
 
-// Rows per thread of the single-image kernel: R = 5 (2 Gaussian halo rows per
-// 5 output rows; 405 CTAs on 1920 x 1080, 1620 on 3840 x 2160), or R = 2 when
-// an image has fewer 128 x 40 tiles than SMs (the most CTAs for a small
-// image).  Measured per launch, back to back, on 640x480 / 1920x1080 /
-// 3840x2160: R = 2 8.2 / 12.8 / 26.6 us, R = 5 12.3 / 12.3 / 24.6 us, R = 15
-// 20.6 / 20.5 / 26.7 us (timer steps of 2.05 us).
-int edge_single_rows(int W, int H, int num_sms) {
-    const long long tiles5 = (long long)((W + TW - 1) / TW) * ((H + 39) / 40);
-    return tiles5 >= (num_sms > 0 ? num_sms : 152) ? 5 : 2;
+// Rows per thread R of the single-image kernel (2 .. 8): a CTA's time grows
+// with its R rows and two more (the Gaussian halo), the launch takes waves of
+// the resident CTAs (6 per SM with Phase, about 10 without), the last one
+// partly filled; the R with the least max(1, waves + 1/2) (R + 2).  Measured back to back (us), R = 2 / 3 / 5 / 6 / 8: 640x480
+// 3.4 / 4.0 / 4.6 / 5.0 / 5.5, 1280x720 4.4 / 5.1 / 6.4 / 6.7 / 7.5, 1920x1080
+// 6.4 / 6.2 / 7.7 / 9.0 / 10.5, 3840x2160 16.5 / 14.8 / 13.5 / 13.1 / 13.4 (the
+// rule picks 2, 2, 3 and 6; R = 5 above 152 tiles of 128 x 40, 2 below, before);
+// gx alone, R = 2 / 5: 1920x1080 3.5 / 3.8, 3840x2160 8.9 / 7.1 (2 and 5 picked).
+int edge_single_rows(int W, int H, bool phase, int num_sms) {
+    const double slots = (phase ? 6.0 : 10.0) * (num_sms > 0 ? num_sms : 152);
+    int best = 2;
+    double best_cost = 1e30;
+    for (int r = 2; r <= 8; ++r) {
+        const double tiles = (double)((W + TW - 1) / TW) * (double)((H + 8 * r - 1) / (8 * r));
+        const double cost = std::max(1.0, tiles / slots + 0.5) * (r + 2);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = r;
+        }
+    }
+    return best;
 }
 
 void edge_tile_dims(int mode, int* tw, int* th) {

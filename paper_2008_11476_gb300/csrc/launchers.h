@@ -29,7 +29,7 @@ constexpr int EDGE_MODE_BINOM5 = 7;
 int edge_mode(const EdgeParams& p);
 void edge_tile_dims(int mode, int* tw, int* th);
 // output rows per thread of the single-image edge kernel for a W x H image
-int edge_single_rows(int W, int H, int num_sms);
+int edge_single_rows(int W, int H, bool phase, int num_sms);
 cudaError_t launch_edge(const CUtensorMap& map, const EdgeParams& p, cudaStream_t s);
 // rows: output rows per thread of the edge kernel's 128 x 8R tiles, R = 5,
 // 10 or EDGE_ROWS (15, the default); the Gaussian kernel keeps its own tile
@@ -57,18 +57,21 @@ int binom5_batch_blocks_per_sm();
 // Harris: the strip kernel (harris_fast_path) or the general one; the tensor map
 // of the group's input must use the box harris_box() gives.
 bool harris_fast_path(const HarrisParams& p);
-int harris_fast_rows(int W, int H, int num_sms);
+// rows per thread and strips per row of a strip-kernel launch over n images;
+// wide_ok: 32 strips are allowed (harris_wide_ok of every image)
+void harris_fast_shape(const int* W, const int* H, int n, bool wide_ok, int num_sms, int* rows,
+                       int* lanes);
+bool harris_wide_ok(const HarrisParams& p);
+void harris_tile(const HarrisParams& p, int* w, int* h);
 void harris_box(const HarrisParams& p, int* w, int* h);
 cudaError_t launch_harris(const CUtensorMap& map, const HarrisParams& p, cudaStream_t s);
 // harris_fast_path groups over n images in one launch (every image's rows
-// equal; tensor maps boxed for them); total = tile_start[n]; resp: some
+// and lanes equal; tensor maps boxed for them); total = tile_start[n]; resp: some
 // image exports its response; borders: some image has harris_borders()
 bool harris_borders(const HarrisParams& p);
 cudaError_t launch_harris_batch(const CUtensorMap* maps, const HarrisParams* ps,
                                 const int* tile_start, const int* tiles_x, int n, int total,
-                                bool tomasi, bool resp, bool borders, cudaStream_t s);
-int harris_fast_tile_w();
-int harris_batch_rows(const int* W, const int* H, int n, int num_sms);
+                                bool tomasi, bool resp, bool borders, int lanes, cudaStream_t s);
 cudaError_t launch_generic(const GenericDesc& d, cudaStream_t s);
 cudaError_t launch_plain(const PlainParams& p, cudaStream_t s);
 cudaError_t launch_eqhist(const EqHistParams& p, cudaStream_t s);

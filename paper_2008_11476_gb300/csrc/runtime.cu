@@ -281,7 +281,7 @@ hvx_status build_edge(Plan& P, Group& G, const EdgeMatch& m, Context* ctx) {
     }
     // one image per launch: R rows per thread, a 160 x (8R + 4) box (the
     // batch kernel encodes its own 160 x EDGE_LOAD_H maps)
-    e.rows = edge_single_rows((int)G.W, (int)G.H, ctx->num_sms);
+    e.rows = edge_single_rows((int)G.W, (int)G.H, e.phase != nullptr, ctx->num_sms);
     if (const char* env = getenv("HVX_EDGE_ROWS")) {  // tuning knob: 2 .. EDGE_ROWS
         const int r = atoi(env);
         static bool said = false;
@@ -328,7 +328,7 @@ hvx_status build_binom5(Plan& P, Group& G, Context* ctx) {
     set_rect(e.valid, op.out->valid);
     // one image per launch: R rows per thread, a 160 x (8R + 4) box (the batch
     // kernel encodes its own 160 x (8R + 4) maps for the R it runs)
-    e.rows = edge_single_rows((int)G.W, (int)G.H, ctx->num_sms);
+    e.rows = gauss_single_rows((int)G.W, (int)G.H, ctx->num_sms);
     return encode_u8_map(&G.tmap, op.in[0], EDGE_LOAD_W, (uint32_t)(8 * e.rows + 4));
 }
 
@@ -465,7 +465,6 @@ hvx_status build_harris(Plan& P, Group& G, const HarrisMatch& m, Context* ctx) {
     h.border_b = s0.node->border;
     h.cval_b = s0.node->cval;
     h.wr = 2;
-    h.rows = harris_fast_rows((int)G.W, (int)G.H, ctx->num_sms > 0 ? ctx->num_sms : 152);
     h.tomasi = m.tomasi ? 1 : 0;
     h.kn = m.tomasi ? 0 : r.node->p.kn;
     h.kd = m.tomasi ? 1 : r.node->p.kd;
@@ -486,6 +485,9 @@ hvx_status build_harris(Plan& P, Group& G, const HarrisMatch& m, Context* ctx) {
         h.thr_f = (float)t.node->p.thr_value;
         if (!m.tomasi) h.q_thr = harris_q_threshold(h.thr_f, h.kd);
     }
+    const int w = (int)G.W, ht = (int)G.H;
+    harris_fast_shape(&w, &ht, 1, harris_wide_ok(h), ctx->num_sms > 0 ? ctx->num_sms : 152, &h.rows,
+                      &h.lanes);
     int bw = 0, bh = 0;
     harris_box(h, &bw, &bh);
     return encode_u8_map(&G.tmap, sx.in[0], bw, bh);
@@ -850,6 +852,7 @@ struct BatchEntry {
     bool harris = false;  // corner batch: one direct launch
     bool tomasi = false;  // ... of the Shi-Tomasi kernel
     bool resp = false;    // ... where some image exports its response
+    int lanes = 16;        // ... with this many strips per row of threads
     bool borders = false;  // ... where some image has a border mode
     std::vector<int> rows;  // edge batch: rows per thread of each image's tiles
     std::vector<void*> more_dmem;  // edge batch split by size class: the other tables
@@ -1209,8 +1212,10 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
         ws[i] = (int)gs[i]->plan.groups[0].W;
         hs[i] = (int)gs[i]->plan.groups[0].H;
     }
-    const int rows = harris_batch_rows(ws.data(), hs.data(), n, ctx->num_sms);
-    const int tw = harris_fast_tile_w();
+    bool wide_ok = true;
+    for (int i = 0; i < n; ++i) wide_ok = wide_ok && harris_wide_ok(gs[i]->plan.groups[0].harris);
+    int rows = 0, lanes = 0, tw = 0, th = 0;
+    harris_fast_shape(ws.data(), hs.data(), n, wide_ok, ctx->num_sms, &rows, &lanes);
     const size_t params_off = (size_t)n * sizeof(CUtensorMap);
     const size_t tiles_off = params_off + (size_t)n * sizeof(HarrisParams);
     const size_t tx_off = tiles_off + (size_t)(n + 1) * sizeof(int);
@@ -1221,6 +1226,8 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
         const Group& G = gs[i]->plan.groups[0];
         HarrisParams hp = G.harris;
         hp.rows = rows;
+        hp.lanes = lanes;
+        harris_tile(hp, &tw, &th);
         int bw = 0, bh = 0;
         harris_box(hp, &bw, &bh);
         CUtensorMap map;
@@ -1229,7 +1236,7 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
         std::memcpy(host.data() + (size_t)i * sizeof(CUtensorMap), &map, sizeof(map));
         std::memcpy(host.data() + params_off + (size_t)i * sizeof(HarrisParams), &hp, sizeof(hp));
         tiles_x[i] = (ws[i] + tw - 1) / tw;
-        tile_start[i + 1] = tile_start[i] + tiles_x[i] * ((hs[i] + 8 * rows - 1) / (8 * rows));
+        tile_start[i + 1] = tile_start[i] + tiles_x[i] * ((hs[i] + th - 1) / th);
     }
     std::memcpy(host.data() + tiles_off, tile_start.data(), (n + 1) * sizeof(int));
     std::memcpy(host.data() + tx_off, tiles_x.data(), n * sizeof(int));
@@ -1249,6 +1256,7 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
     for (int i = 0; i < n; ++i) out.plan_ids[i] = gs[i]->plan_id;
     out.dmem = dmem;
     out.harris = true;
+    out.lanes = lanes;
     out.tomasi = gs[0]->plan.groups[0].harris.tomasi != 0;
     out.resp = false;
     for (int i = 0; i < n; ++i) {
@@ -1374,7 +1382,8 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             reinterpret_cast<const CUtensorMap*>(base),
             reinterpret_cast<const HarrisParams*>(base + params_off),
             reinterpret_cast<const int*>(base + tiles_off), reinterpret_cast<const int*>(base + tx_off),
-            hit->n, hit->total_tiles, hit->tomasi, hit->resp, hit->borders, s));
+            hit->n, hit->total_tiles, hit->tomasi, hit->resp, hit->borders, hit->lanes,
+            s));
     }
     return cuda_status(cudaGraphLaunch(hit->exec, s));
 }
