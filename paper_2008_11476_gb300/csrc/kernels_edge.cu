@@ -1004,20 +1004,21 @@ int edge_mode(const EdgeParams& p) {
 }
 
 // Rows per thread R of the single-image kernel (2 .. 8): a CTA's time grows
-// with its R rows and two more (the Gaussian halo), the launch takes waves of
-// the resident CTAs (6 per SM with Phase, about 10 without), the last one
-// partly filled; the R with the least max(1, waves + 1/2) (R + 2).  Measured back to back (us), R = 2 / 3 / 5 / 6 / 8: 640x480
-// 3.4 / 4.0 / 4.6 / 5.0 / 5.5, 1280x720 4.4 / 5.1 / 6.4 / 6.7 / 7.5, 1920x1080
-// 6.4 / 6.2 / 7.7 / 9.0 / 10.5, 3840x2160 16.5 / 14.8 / 13.5 / 13.1 / 13.4 (the
-// rule picks 2, 2, 3 and 6; R = 5 above 152 tiles of 128 x 40, 2 below, before);
-// gx alone, R = 2 / 5: 1920x1080 3.5 / 3.8, 3840x2160 8.9 / 7.1 (2 and 5 picked).
+// with its R rows and the halo's, the launch takes waves of the resident CTAs
+// (6 per SM with Phase, about 10 without), the last one partly filled; the R
+// with the least max(1, waves + 1/2) (R + 2.5).  Measured back to back (us), R
+// = 2 / 3 / 5 / 6 / 8: 640x480 3.4 / 4.0 / 4.6 / 5.0 / 5.5, 1280x720 4.4 / 5.1
+// / 6.4 / 6.7 / 7.5, 1920x1080 6.4 / 6.2 / 7.7 / 9.0 / 10.5, 3840x2160 16.5 /
+// 14.8 / 13.5 / 13.1 / 13.4 (the rule picks 2, 2, 3 and 6; R = 5 above 152
+// tiles of 128 x 40, 2 below, before); gx alone, R = 2 / 5: 1920x1080 3.5 /
+// 3.8, 3840x2160 8.9 / 7.1 (2 and 5 picked).
 int edge_single_rows(int W, int H, bool phase, int num_sms) {
     const double slots = (phase ? 6.0 : 10.0) * (num_sms > 0 ? num_sms : 152);
     int best = 2;
     double best_cost = 1e30;
     for (int r = 2; r <= 8; ++r) {
         const double tiles = (double)((W + TW - 1) / TW) * (double)((H + 8 * r - 1) / (8 * r));
-        const double cost = std::max(1.0, tiles / slots + 0.5) * (r + 2);
+        const double cost = std::max(1.0, tiles / slots + 0.5) * (r + 2.5);
         if (cost < best_cost) {
             best_cost = cost;
             best = r;
