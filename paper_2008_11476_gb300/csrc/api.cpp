@@ -122,6 +122,7 @@ bool valid_fmt(int f) { return f >= HVX_DF_U8 && f <= HVX_DF_UYVY; }
 
 void destroy_image(Image* im) {
     if (im->dev && im->owns_mem) im->ctx->pool.free(im->dev);
+    if (im->mirror) im->ctx->host.free(im->mirror, im->mirror_bytes);
     im->magic = 0;
     delete im;
 }
@@ -279,7 +280,6 @@ hvx_status hvxReleaseContext(hvx_context* pc) {
     for (Image* im : images) destroy_image(im);
     c->images.clear();
     destroy_batch_cache(c);
-    if (c->d_error) cudaFree(c->d_error);
     for (cudaEvent_t e : c->io_events) cudaEventDestroy(e);
     if (c->io_in) cudaStreamDestroy(c->io_in);
     if (c->io_out) cudaStreamDestroy(c->io_out);
@@ -681,6 +681,7 @@ hvx_status hvxWaitGraph(hvx_graph hg) {
     cudaError_t e = cudaEventSynchronize(g->done);
     g->scheduled = false;
     if (e != cudaSuccess) return set_last(g, cuda_status(e));
+    g->settled = true;
     return set_last(g, check_device_error(g->ctx));
 }
 
@@ -1139,14 +1140,23 @@ hvx_status hvxGetNodeResult(hvx_node hn, void* out, uint64_t size) {
     if (n->graph->ctx->plan_only) return HVX_ERROR_NOT_SUPPORTED;
     Image* r = n->out[0];
     if (!r || !r->dev) return HVX_ERROR_NOT_VERIFIED;
+    // the host's copy where the plan writes one: no copy, and no wait when the
+    // graph has been waited for (else for the default stream's work, as a
+    // synchronous copy does)
+    auto fetch = [&](void* to, uint64_t bytes) {
+        if (!r->mirror_live) return cudaMemcpy(to, r->dev, bytes, cudaMemcpyDeviceToHost);
+        cudaError_t e = n->graph->settled ? cudaSuccess : cudaStreamSynchronize(cudaStreamLegacy);
+        if (e == cudaSuccess) std::memcpy(to, r->mirror, bytes);
+        return e;
+    };
     if (n->kind == N_HIST) {
         const uint64_t bytes = 4ull * (uint64_t)n->p.hist_bins;
         if (size < bytes) return HVX_ERROR_INVALID_PARAMETERS;
-        return cuda_status(cudaMemcpy(out, r->dev, bytes, cudaMemcpyDeviceToHost));
+        return cuda_status(fetch(out, bytes));
     }
     uint64_t w[4] = {0, 0, 0, 0};
     const uint64_t bytes = n->kind == N_MEANSTD ? 24 : 32;
-    cudaError_t e = cudaMemcpy(w, r->dev, bytes, cudaMemcpyDeviceToHost);
+    cudaError_t e = fetch(w, bytes);
     if (e != cudaSuccess) return cuda_status(e);
     if (n->kind == N_MEANSTD) {
         if (size < sizeof(hvx_mean_stddev)) return HVX_ERROR_INVALID_PARAMETERS;

@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -174,6 +175,8 @@ struct JitKernel {
     // form where the group has one
     bool strips = false;
     StripPlan strip;
+    // resident CTAs per SM of fn_batch by rows per thread (0: not asked yet)
+    mutable std::array<std::atomic<int>, 25> per_sm{};
     // the group's images: halo, and whether it is an external input
     int n_buf = 0;
     std::array<int, HVX_JIT_MAX_BUF> halo{};
@@ -1649,15 +1652,25 @@ int set_tiles(const JitKernel& k, HvxJitParams& p, unsigned* gx, unsigned* gy) {
     return p.rows ? strip_smem_bytes(k.strip, p.rows) : k.smem_bytes;
 }
 
+// Resident CTAs per SM of the strip kernels with `rows` rows per thread.
+int strip_ctas_per_sm(const JitKernel& k, int rows) {
+    std::atomic<int>& known = k.per_sm[rows];
+    int per = known.load(std::memory_order_relaxed);
+    if (per > 0) return per;
+    if (!k.fn_batch || driver().occupancy(&per, k.fn_batch, STRIP_THREADS,
+                                          (size_t)strip_smem_bytes(k.strip, rows)) != CUDA_SUCCESS)
+        return 5;
+    per = std::max(per, 1);
+    known.store(per, std::memory_order_relaxed);
+    return per;
+}
+
 // CTAs of an image with global operators: its share (by tiles) of the CTAs that
 // are resident at a time, so that each commits one partial result.
 int reduction_ctas(const JitKernel& k, const HvxJitParams& p, long long tiles, long long all,
                    int num_sms) {
-    int per = 5;
-    if (k.fn && driver().occupancy(&per, k.fn, STRIP_THREADS,
-                                   (size_t)strip_smem_bytes(k.strip, p.rows)) != CUDA_SUCCESS)
-        per = 5;
-    const long long share = ((long long)std::max(per, 1) * num_sms * tiles + all - 1) / all;
+    const long long slots = (long long)strip_ctas_per_sm(k, p.rows) * num_sms;
+    const long long share = (slots * tiles + all - 1) / all;
     return (int)std::max(1ll, std::min({tiles, share, (long long)STRIP_MAX_CTAS}));
 }
 
@@ -1700,16 +1713,11 @@ int strip_rows(const JitKernel& k, const int* W, const int* H, int n, int num_sm
     int best = u;
     double best_cost = 1e30;
     for (int r = u; r <= 24; r += u) {
-        const int smem = strip_smem_bytes(k.strip, r);
-        if (smem > kStripSmem) break;
-        int per = 5;
-        if (k.fn_batch && driver().occupancy(&per, k.fn_batch, STRIP_THREADS, (size_t)smem) !=
-                              CUDA_SUCCESS)
-            per = 5;
+        if (strip_smem_bytes(k.strip, r) > kStripSmem) break;
         long long tiles = 0;
         for (int i = 0; i < n; ++i)
             tiles += (long long)((W[i] + STRIP_TW - 1) / STRIP_TW) * ((H[i] + 8 * r - 1) / (8 * r));
-        const double waves = (double)tiles / ((double)std::max(per, 1) * num_sms);
+        const double waves = (double)tiles / ((double)strip_ctas_per_sm(k, r) * num_sms);
         const double cost = std::max(1.0, waves + 0.5) * (r + 0.3 * pro + 1.0);
         if (cost < best_cost) {
             best_cost = cost;
@@ -1738,7 +1746,7 @@ std::string shape_key(const GenericDesc& d, const std::vector<std::string>& user
         c.in[e].ptr = c.out[e].ptr = nullptr;
         c.in[e].pitch = c.out[e].pitch = 0;
     }
-    for (int k = 0; k < c.n_stage; ++k) c.st[k].res = nullptr;
+    for (int k = 0; k < c.n_stage; ++k) c.st[k].res = c.st[k].mirror = nullptr;
     std::string key(reinterpret_cast<const char*>(&c), sizeof(c));
     key += std::to_string(device);
     for (const char* n : {"HVX_CODEGEN_TMA", "HVX_CODEGEN_ROWS", "HVX_CODEGEN_COLS",
@@ -1831,6 +1839,7 @@ bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code
     for (int k = 0; k < d.n_stage; ++k)
         if (op_is_global(d.st[k].op)) {
             if (nres >= HVX_JIT_MAX_RES) return false;
+            p.mirror[nres] = d.st[k].mirror;
             p.res[nres++] = d.st[k].res;
         }
     int num_sms = 152;

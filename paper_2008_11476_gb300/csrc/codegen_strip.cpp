@@ -1070,11 +1070,15 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
         for (size_t j = 0; j < globals.size(); ++j) {
             const int k = globals[j];
             const std::string res = "p.res[" + std::to_string(j) + "]",
+                              mir = "p.mirror[" + std::to_string(j) + "]",
                               scr = "((unsigned char*)" + res + " + " +
                                     std::to_string(scratch_at(k) + 16) + ")";
             if (d.st[k].op == OP_MEANSTD) {
-                o << "  if (threadIdx.x < 3)\n    ((unsigned long long*)" << res
-                  << ")[threadIdx.x] = atomicExch((unsigned long long*)" << scr << " + threadIdx.x, 0ull);\n";
+                o << "  if (threadIdx.x < 3) {\n    const unsigned long long v = atomicExch((unsigned long "
+                     "long*)"
+                  << scr << " + threadIdx.x, 0ull);\n    ((unsigned long long*)" << res
+                  << ")[threadIdx.x] = v;\n    if (" << mir << ") ((unsigned long long*)" << mir
+                  << ")[threadIdx.x] = v;\n  }\n";
             } else if (d.st[k].op == OP_MINMAX) {
                 o << "  {\n    HvxMinMaxAcc a;\n    hvx_mm_init(a);\n"
                   << "    const int* const q = (const int*)" << scr << ";\n"
@@ -1082,10 +1086,14 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
                   << "      hvx_mm_merge(a, __ldcg(q + 6 * i), __ldcg(q + 6 * i + 2), __ldcg(q + 6 * i + 4), "
                      "__ldcg(q + 6 * i + 1), __ldcg(q + 6 * i + 3), __ldcg(q + 6 * i + 5));\n"
                   << "    hvx_mm_block<" << warps << ">(a, smm);\n"
-                  << "    if (threadIdx.x == 0) hvx_mm_result((unsigned long long*)" << res << ", a);\n  }\n";
+                  << "    if (threadIdx.x == 0) {\n      hvx_mm_result((unsigned long long*)" << res
+                  << ", a);\n      if (" << mir << ") hvx_mm_result((unsigned long long*)" << mir
+                  << ", a);\n    }\n  }\n";
             } else {
                 o << "  for (int i = threadIdx.x; i < " << d.st[k].i0 << "; i += " << STRIP_THREADS
-                  << ") ((unsigned*)" << res << ")[i] = atomicExch((unsigned*)" << scr << " + i, 0u);\n";
+                  << ") {\n    const unsigned v = atomicExch((unsigned*)" << scr
+                  << " + i, 0u);\n    ((unsigned*)" << res << ")[i] = v;\n    if (" << mir
+                  << ") ((unsigned*)" << mir << ")[i] = v;\n  }\n";
             }
         }
         o << "  if (threadIdx.x == 0) *done = 0u;\n}\n\n"

@@ -66,6 +66,24 @@ class DevicePool {
     std::multimap<uint64_t, void*> cache_;
 };
 
+// A context's page-locked host memory that kernels write directly: the error
+// word and the results of global operators, so that reading them after a wait
+// takes no copy.  One 64 KB block per context, handed out in 64-byte steps
+// (verification and release only: one host thread at a time); its work is done
+// when the context is released, so the next context may take the block over.
+class HostBlock {
+  public:
+    ~HostBlock();
+    bool alloc(uint64_t bytes, void** host, void** dev);  // false when it is full
+    void free(void* host, uint64_t bytes);
+
+  private:
+    static constexpr uint64_t kBytes = 64 * 1024, kStep = 64;
+    uint8_t* host_ = nullptr;
+    uint8_t* dev_ = nullptr;
+    std::vector<bool> used_;
+};
+
 struct Context;
 struct Graph;
 struct Server;
@@ -92,6 +110,12 @@ struct Image {
     // non-virtual data vertex of the graph owned by it, with no pixels; dev
     // holds the device result block.
     bool is_result = false;
+    // A result's copy in host memory that the device writes (HostBlock), and
+    // whether the graph's plan writes it.
+    void* mirror = nullptr;
+    void* mirror_dev = nullptr;
+    uint64_t mirror_bytes = 0;
+    bool mirror_live = false;
 };
 
 // Internal format of result images.
@@ -270,6 +294,7 @@ struct Graph {
     Plan plan;
     cudaEvent_t done = nullptr;
     bool scheduled = false;
+    bool settled = false;        // nothing launched since the last wait for the graph
     cudaStream_t last_stream = nullptr;
     std::atomic<int> busy{0};  // in flight on a server
 };
@@ -284,7 +309,10 @@ struct Context {
     std::vector<Image*> images;  // non-virtual images
     std::vector<Graph*> graphs;
     std::vector<Server*> servers;
-    int* d_error = nullptr;      // device error word (bounded waits that ran out)
+    HostBlock host;
+    // error word (bounded waits that ran out): its device address, and the host's
+    int* d_error = nullptr;
+    volatile int* h_error = nullptr;
     int num_sms = 0;
     BatchCache* batch = nullptr;
     // hvxScheduleGraphBatchHost: copy streams and events of its pipeline

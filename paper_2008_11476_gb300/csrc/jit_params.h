@@ -25,7 +25,8 @@ struct HvxJitParams {
     void* out[HVX_JIT_MAX_EXT];     // external outputs
     unsigned long long out_pitch[HVX_JIT_MAX_EXT];
     void* res[HVX_JIT_MAX_RES];     // result blocks of the group's global operators
-    int* err;                       // device error word (a bounded wait that ran out)
+    void* mirror[HVX_JIT_MAX_RES];  // strip form: host copies of the results (may be null)
+    int* err;                       // error word (a bounded wait that ran out)
     int rows;                       // strip form: output rows per thread (tiles of 128 x 8 rows)
     int ctas;                       // strip form with global operators: CTAs of this image
     HvxTensorMap tmap[HVX_JIT_MAX_EXT];  // inputs staged by TMA: box = the staged slot (tile

@@ -112,6 +112,7 @@ struct GenStage {
     float f0, f1;      // F32 thresholds
     int64_t k0, k1;    // integer thresholds, or kn / kd of the Harris response
     void* res;         // global operators: device result block (out is -1)
+    void* mirror;      // ... and its host copy that the device writes (may be null)
 };
 
 struct GenExt {

@@ -618,6 +618,7 @@ hvx_status build_generic(Plan& P, Group& G) {
         for (int k = 0; k < op.n_in; ++k) st.in[k] = buf[op.in[k]];
         st.out = op.out->is_result ? -1 : buf[op.out];
         st.res = op.out->is_result ? op.out->dev : nullptr;
+        st.mirror = op.out->is_result ? op.out->mirror_dev : nullptr;
         st.rx = op.rx;
         st.ry = op.ry;
         st.rounding = op.node->rounding;
@@ -667,14 +668,85 @@ hvx_status build_generic(Plan& P, Group& G) {
 
 }  // namespace
 
+namespace {
+
+// Page-locked blocks of released contexts, for the next ones (allocating and
+// freeing one takes some 260 us): at most kMost are kept.
+struct HostBlockPool {
+    static constexpr size_t kMost = 8;
+    std::mutex mu;
+    std::vector<void*> blocks;
+};
+HostBlockPool& host_blocks() {
+    static auto* p = new HostBlockPool();
+    return *p;
+}
+
+}  // namespace
+
+HostBlock::~HostBlock() {
+    if (!host_) return;
+    {
+        HostBlockPool& p = host_blocks();
+        std::lock_guard<std::mutex> lk(p.mu);
+        if (p.blocks.size() < HostBlockPool::kMost) {
+            p.blocks.push_back(host_);
+            return;
+        }
+    }
+    cudaFreeHost(host_);
+}
+
+bool HostBlock::alloc(uint64_t bytes, void** host, void** dev) {
+    if (!host_) {
+        void *h = nullptr, *d = nullptr;
+        {
+            HostBlockPool& p = host_blocks();
+            std::lock_guard<std::mutex> lk(p.mu);
+            if (!p.blocks.empty()) {
+                h = p.blocks.back();
+                p.blocks.pop_back();
+            }
+        }
+        if ((!h && cudaHostAlloc(&h, kBytes, cudaHostAllocMapped | cudaHostAllocPortable) !=
+                       cudaSuccess) ||
+            cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+            cudaGetLastError();
+            if (h) cudaFreeHost(h);
+            return false;
+        }
+        std::memset(h, 0, kBytes);
+        host_ = static_cast<uint8_t*>(h);
+        dev_ = static_cast<uint8_t*>(d);
+        used_.assign(kBytes / kStep, false);
+    }
+    const size_t n = (size_t)((bytes + kStep - 1) / kStep);
+    for (size_t a = 0, run = 0; a < used_.size(); ++a) {
+        run = used_[a] ? 0 : run + 1;
+        if (run == n) {
+            const size_t first = a + 1 - n;
+            for (size_t k = first; k <= a; ++k) used_[k] = true;
+            *host = host_ + first * kStep;
+            *dev = dev_ + first * kStep;
+            return true;
+        }
+    }
+    return false;
+}
+
+void HostBlock::free(void* host, uint64_t bytes) {
+    const size_t first = (size_t)(static_cast<uint8_t*>(host) - host_) / kStep;
+    const size_t n = (size_t)((bytes + kStep - 1) / kStep);
+    for (size_t k = first; k < first + n && k < used_.size(); ++k) used_[k] = false;
+}
+
 hvx_status ensure_context_device_state(Context* ctx) {
     if (!ctx->d_error) {
-        cudaError_t e = cudaMalloc(&ctx->d_error, sizeof(int));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return HVX_ERROR_NO_MEMORY;
-        }
-        if (cudaMemset(ctx->d_error, 0, sizeof(int)) != cudaSuccess) return HVX_ERROR_DEVICE;
+        void *h = nullptr, *d = nullptr;
+        if (!ctx->host.alloc(sizeof(int), &h, &d)) return HVX_ERROR_NO_MEMORY;
+        ctx->h_error = static_cast<volatile int*>(h);
+        *ctx->h_error = 0;
+        ctx->d_error = static_cast<int*>(d);
     }
     if (!ctx->num_sms) {
         cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
@@ -683,14 +755,10 @@ hvx_status ensure_context_device_state(Context* ctx) {
     return HVX_SUCCESS;
 }
 
+// After a wait for the work in question.
 hvx_status check_device_error(Context* ctx) {
-    int v = 0;
-    if (cudaMemcpy(&v, ctx->d_error, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) {
-        cudaGetLastError();
-        return HVX_ERROR_DEVICE;
-    }
-    if (v == 0) return HVX_SUCCESS;
-    cudaMemset(ctx->d_error, 0, sizeof(int));
+    if (*ctx->h_error == 0) return HVX_SUCCESS;
+    *ctx->h_error = 0;
     return HVX_ERROR_TIMEOUT;
 }
 
@@ -713,6 +781,10 @@ hvx_status alloc_results(Plan& P, Context* ctx) {
                 op.out->bytes = n;
                 cudaMemset(op.out->dev, 0, n);
                 cudaMemset(op.out->dev, global_result_fill(op.kind), res);
+            }
+            if (!op.out->mirror && ctx->host.alloc(res, &op.out->mirror, &op.out->mirror_dev)) {
+                op.out->mirror_bytes = res;
+                std::memset(op.out->mirror, global_result_fill(op.kind), res);
             }
         }
         if (op.kind == OP_EQHIST && !op.node->d_aux) {
@@ -797,8 +869,12 @@ hvx_status prepare_launches(Graph* g) {
                 G.jit_on = jit_prepare(G.gdesc, G.user_code, !ctx->plan_only, ctx->device, &G.jit,
                                        &why);
                 G.jit.p.err = ctx->d_error;
-                // the strip form's last CTA writes the whole result
-                if (G.jit_on && G.jit.p.rows > 0) G.resets.clear();
+                // the strip form's last CTA writes the whole result, and its mirror
+                const bool strips = G.jit_on && G.jit.p.rows > 0;
+                if (strips) G.resets.clear();
+                for (int i : G.ops)
+                    if (op_is_global(P.ops[i].kind))
+                        P.ops[i].out->mirror_live = strips && P.ops[i].out->mirror;
                 if (!G.jit_on && getenv("HVX_CODEGEN_VERBOSE"))
                     fprintf(stderr, "hvx: no generated kernel for a group: %s\n", why.c_str());
                 if (!G.jit_on && (must_gen || user))
@@ -814,6 +890,7 @@ hvx_status prepare_launches(Graph* g) {
 hvx_status launch_plan(Graph* g, cudaStream_t s) {
     if (fault_fires(HVX_FAULT_LAUNCH)) return HVX_ERROR_DEVICE;  // injected, nothing enqueued
     bind_device(g->ctx);
+    g->settled = false;
     for (Group& G : g->plan.groups) {
         NvtxRange nvtx(G.jit_on ? "hvx launch generated" : group_kernel_name(G.kernel));
         cudaError_t e = cudaSuccess;
@@ -1329,6 +1406,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
         }
         return HVX_SUCCESS;
     }
+    for (int i = 0; i < n; ++i) gs[i]->settled = false;
     if (!ctx->batch) ctx->batch = new BatchCache();
     BatchCache* bc = ctx->batch;
     BatchEntry* hit = nullptr;
