@@ -1374,24 +1374,30 @@ __device__ __forceinline__ void hvx_cols(unsigned (&w)[NW], int x, int W, unsign
             const std::string E_ = std::to_string(e);
             const std::string ld = "hvx_ld<" + std::to_string(d.in[e].fmt) + ">(p.in[" + E_ +
                                    "], p.in_pitch[" + E_ + "], ";
-            const char* at = fill == FILL_MIRROR   ? "hvx_mirror(x, W), hvx_mirror(y, H))"
-                             : fill == FILL_REPEAT ? "hvx_repeat(x, W), hvx_repeat(y, H))"
-                                                   : "min(max(x, 0), W - 1), min(max(y, 0), H - 1))";
+            // (the nearest pixel lies in the box: every tile reaches into the image)
+            const char* at = fill == FILL_MIRROR ? "hvx_mirror(x, W), hvx_mirror(y, H))"
+                                                 : "hvx_repeat(x, W), hvx_repeat(y, H))";
+            const std::string near_x = "min(max(x, 0), W - 1)", near_y = "min(max(y, 0), H - 1)";
             o << "__device__ void hvx_fill" << i
               << "(const HvxJitParams& p, unsigned char* box, int x0, int y0, int R) {\n"
-              << "  const int W = p.W, H = p.H, h = " << h << ";\n"
+              << "  const int W = p.W, H = p.H;\n  constexpr int h = " << h << ";\n"
               << "  const int c0 = x0 - h, c1 = min(x0 + " << STRIP_TW << ", W) + h;\n"
               << "  const int r0 = y0 - h, r1 = min(y0 + 8 * R, H) + h;\n"
-              << "  const int lane = threadIdx.x & 31, left = max(0, min(c1, 0) - c0), right = max(c0, W);\n"
-              << "  for (int y = r0 + (int)(threadIdx.x >> 5); y < r1; y += " << STRIP_THREADS / 32
-              << ") {\n"
-              << "    const bool in = y >= 0 && y < H;\n"
-              << "    const int n = in ? left + max(0, c1 - right) : c1 - c0;\n"
-              << "    for (int k = lane; k < n; k += 32) {\n"
-              << "      const int x = !in || k < left ? c0 + k : right + k - left;\n"
-              << "      box[(y - r0) * " << STRIP_BOX_W << " + x - x0 + 16] = (unsigned char)"
-              << (fill == FILL_CONSTANT ? std::to_string(d.buf[b].cval) + "u" : ld + at) << ";\n"
-              << "    }\n  }\n}\n";
+              << "  auto put = [&](int x, int y) {\n"
+              << "    box[(y - r0) * " << STRIP_BOX_W << " + x - x0 + 16] = (unsigned char)"
+              << (fill == FILL_CONSTANT    ? std::to_string(d.buf[b].cval) + "u"
+                  : fill == FILL_REPLICATE ? "box[(" + near_y + " - r0) * " + std::to_string(STRIP_BOX_W) +
+                                                 " + " + near_x + " - x0 + 16]"
+                                           : ld + at)
+              << ";\n  };\n"
+              << "  // rows above and below the image, then the sides of the rows inside\n"
+              << "  #pragma unroll 1\n  for (int k = 1; k <= h; ++k)\n"
+              << "    for (int x = c0 + (int)threadIdx.x; x < c1; x += " << STRIP_THREADS << ") {\n"
+              << "      if (-k >= r0) put(x, -k);\n      if (H - 1 + k < r1) put(x, H - 1 + k);\n    }\n"
+              << "  const int ra = max(r0, 0), rb = min(r1, H);\n"
+              << "  for (int i = threadIdx.x; i < (rb - ra) * h; i += " << STRIP_THREADS << ") {\n"
+              << "    const int y = ra + i / h, k = i % h + 1;\n"
+              << "    if (-k >= c0) put(-k, y);\n    if (W - 1 + k < c1) put(W - 1 + k, y);\n  }\n}\n";
         }
         // the boxes of one stage, their loads, and one tile on them
         const bool boxed = !boxes.empty();

@@ -234,6 +234,27 @@ __device__ __forceinline__ void for_each_outside(int R, int C, int bx, int by, i
     }
 }
 
+// Calls f(x, y) for the pixels outside the W x H image within HALO of it that a
+// tw x th tile at (x0, y0) with that halo covers, spread over the CTA's
+// threads (rows above and below with their corners, then the sides): all that a
+// stencil of radius HALO reads outside the image.
+template <int HALO, class F>
+__device__ __forceinline__ void for_each_ring(int x0, int y0, int tw, int th, int W, int H, F f) {
+    const int c0 = x0 == 0 ? -HALO : x0 - HALO, c1 = min(x0 + tw, W) + HALO;
+    const int r0 = max(y0 - HALO, 0), r1 = min(y0 + th + HALO, H);  // rows inside the image
+#pragma unroll
+    for (int k = 1; k <= HALO; ++k)
+        for (int x = c0 + (int)threadIdx.x; x < c1; x += blockDim.x) {
+            if (y0 == 0) f(x, -k);
+            if (H - 1 + k < y0 + th + HALO) f(x, H - 1 + k);
+        }
+    for (int i = threadIdx.x; i < (r1 - r0) * HALO; i += blockDim.x) {
+        const int y = r0 + i / HALO, k = i % HALO + 1;
+        if (x0 == 0) f(-k, y);
+        if (W - 1 + k < c1) f(W - 1 + k, y);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // 16-bit-lane (SWAR) helpers of the U8 stencil kernels: two pixels per
 // 32-bit word, so that one add or shift works on both.

@@ -61,21 +61,20 @@ __device__ __forceinline__ bool tile_is_interior(const EdgeParams& p, int x0, in
     return x0 >= 1 && y0 >= 1 && x0 + TW + 1 <= (int)p.W && y0 + th + 1 <= (int)p.H;
 }
 
-// Box cells outside the image under REPLICATE / CONSTANT (edge tiles only);
-// lh: the box rows the TMA filled.
-__device__ void fix_box_border(Box& in, const EdgeParams& p, int x0, int y0, int lh) {
+// Box cells outside the image under REPLICATE / CONSTANT that the tile's
+// outputs read (edge tiles only); th: the tile's rows.
+__device__ void fix_box_border(Box& in, const EdgeParams& p, int x0, int y0, int th) {
     const int W = p.W, H = p.H;
     if (p.border_g == HVX_BORDER_UNDEFINED) return;
     const bool cst = p.border_g == HVX_BORDER_CONSTANT;
     const uint8_t cv = (uint8_t)p.cval_g;
-    for_each_outside(lh, LW, x0 - 16, y0 - 1, W, H, [&](int r, int c) {
-        const int x = x0 - 16 + c, y = y0 - 1 + r;
-        in[r][c] = cst ? cv : in[clampi(y, 0, H - 1) - (y0 - 1)][clampi(x, 0, W - 1) - (x0 - 16)];
+    for_each_ring<1>(x0, y0, TW, th, W, H, [&](int x, int y) {
+        in[y - y0 + 1][x - x0 + 16] =
+            cst ? cv : in[clampi(y, 0, H - 1) - (y0 - 1)][clampi(x, 0, W - 1) - (x0 - 16)];
     });
 }
 
-// fix_box_border restricted to box rows r0 .. r1 - 1 and the columns the
-// strips read (12 .. 147), for the batch kernel, whose warps run ahead of
+// fix_box_border restricted to box rows r0 .. r1 - 1, for the batch kernel, whose warps run ahead of
 // each other without a block barrier: each warp fixes the rows its two row
 // groups read, lanes striding over the cells, then syncs.  Neighbouring
 // warps share halo rows; both write the same values, each taken from a cell
@@ -90,20 +89,19 @@ __device__ void fix_box_border_warp(Box& in, const EdgeParams& p, int x0, int y0
     auto put = [&](int r, int c) {
         in[r][c] = cst ? cv : in[clampi(by + r, 0, H - 1) - by][clampi(bx + c, 0, W - 1) - bx];
     };
-    constexpr int C0 = 12, C1 = 148;
+    // columns x0 - 1 .. x0 + TW, one past the image at most
+    const int c0 = 15, c1 = min(16 + TW + 1, W - bx + 1);
     const int ra = max(r0, -by), rb = min(r1, H - by);  // rows inside the image
-    // rows outside the image: every column
-    for (int r = r0; r < r1; ++r)
-        if (r < ra || r >= rb)
-            for (int c = C0 + lane; c < C1; c += 32) put(r, c);
-    // rows inside: the columns left and right of the image
-    const int la = C0, lb = min(C1, -bx), rca = max(C0, W - bx), rcb = C1;
-    const int nl = max(lb - la, 0), nr = max(rcb - rca, 0), n = nl + nr;
-    if (n > 0)
-        for (int i = lane; i < (rb - ra) * n; i += 32) {
-            const int r = ra + i / n, j = i - (i / n) * n;
-            put(r, j < nl ? la + j : rca + j - nl);
-        }
+    // the rows just above and below the image
+    if (-by - 1 >= r0)
+        for (int c = c0 + lane; c < c1; c += 32) put(-by - 1, c);
+    if (H - by >= r0 && H - by < r1)
+        for (int c = c0 + lane; c < c1; c += 32) put(H - by, c);
+    // rows inside: the columns just left and right of the image
+    for (int r = ra + lane; r < rb; r += 32) {
+        if (x0 == 0) put(r, 15);
+        if (W - bx < c1) put(r, W - bx);
+    }
     __syncwarp();
 }
 
@@ -217,7 +215,7 @@ __global__ void __launch_bounds__(GAUSS_THREADS)
     if (__syncthreads_or(!mbar_wait_bounded(&sm.bar[0], 0, p.err))) return;
     const bool interior = tile_is_interior(p, x0, y0, 8 * R);
     if (!interior) {
-        fix_box_border(sm.in[0].b, p, x0, y0, 8 * R + 2);
+        fix_box_border(sm.in[0].b, p, x0, y0, 8 * R);
         __syncthreads();
     }
     gauss_tile<R>(sm.in[0].b, p, x0, y0, interior);

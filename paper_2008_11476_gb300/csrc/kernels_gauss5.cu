@@ -64,35 +64,42 @@ __device__ __forceinline__ uint8_t border_cell(const Box& in, const EdgeParams& 
     return in[clampi(by + r, 0, (int)p.H - 1) - by][clampi(bx + c, 0, (int)p.W - 1) - bx];
 }
 
-// Every box cell outside the image, rows 0 .. lh - 1 (single-image kernel:
-// the whole CTA, then a barrier).
-__device__ void fix_border5(Box& in, const EdgeParams& p, int x0, int y0, int lh) {
+// The box cells outside the image that the tile's outputs read (single-image
+// kernel: the whole CTA, then a barrier); th: the tile's rows.
+__device__ void fix_border5(Box& in, const EdgeParams& p, int x0, int y0, int th) {
     if (p.border_g == HVX_BORDER_UNDEFINED) return;
     const int W = p.W, H = p.H, bx = x0 - 16, by = y0 - 2;
-    for_each_outside(lh, LW, bx, by, W, H,
-                     [&](int r, int c) { in[r][c] = border_cell(in, p, bx, by, r, c); });
+    for_each_ring<2>(x0, y0, TW, th, W, H, [&](int x, int y) {
+        in[y - by][x - bx] = border_cell(in, p, bx, by, y - by, x - bx);
+    });
 }
 
-// The same for box rows r0 .. r1 - 1 and the columns the strips read
-// (12 .. 147), by one warp, lanes striding over the cells (batch kernel:
-// each warp fixes the rows its two row groups read; neighbouring warps write
-// the same values into their shared halo rows).
+// The same for box rows r0 .. r1 - 1, by one warp, lanes striding over the
+// cells (batch kernel: each warp fixes the rows its two row groups read;
+// neighbouring warps write the same values into their shared halo rows).
 __device__ void fix_border5_warp(Box& in, const EdgeParams& p, int x0, int y0, int r0, int r1) {
     if (p.border_g == HVX_BORDER_UNDEFINED) return;
     const int W = p.W, H = p.H, bx = x0 - 16, by = y0 - 2;
     const int lane = threadIdx.x & 31;
-    constexpr int C0 = 12, C1 = 148;
+    auto put = [&](int r, int c) { in[r][c] = border_cell(in, p, bx, by, r, c); };
+    // columns x0 - 2 .. x0 + TW + 1, two past the image at most
+    const int c0 = 14, c1 = min(16 + TW + 2, W - bx + 2);
     const int ra = max(r0, -by), rb = min(r1, H - by);  // rows inside the image
-    for (int r = r0; r < r1; ++r)
-        if (r < ra || r >= rb)
-            for (int c = C0 + lane; c < C1; c += 32) in[r][c] = border_cell(in, p, bx, by, r, c);
-    const int la = C0, lb = min(C1, -bx), rca = max(C0, W - bx);
-    const int nl = max(lb - la, 0), nr = max(C1 - rca, 0), n = nl + nr;
-    if (n > 0)
-        for (int i = lane; i < (rb - ra) * n; i += 32) {
-            const int r = ra + i / n, j = i - (i / n) * n;
-            const int c = j < nl ? la + j : rca + j - nl;
-            in[r][c] = border_cell(in, p, bx, by, r, c);
+    // the two rows above and below the image
+#pragma unroll
+    for (int k = 1; k <= 2; ++k) {
+        const int above = -by - k, below = H - by + k - 1;
+        if (above >= r0 && above < r1)
+            for (int c = c0 + lane; c < c1; c += 32) put(above, c);
+        if (below >= r0 && below < r1)
+            for (int c = c0 + lane; c < c1; c += 32) put(below, c);
+    }
+    // rows inside: the two columns left and right of the image
+    for (int r = ra + lane; r < rb; r += 32)
+#pragma unroll
+        for (int k = 1; k <= 2; ++k) {
+            if (x0 == 0) put(r, 16 - k);
+            if (W - bx + k - 1 < c1) put(r, W - bx + k - 1);
         }
     __syncwarp();
 }
@@ -197,7 +204,7 @@ __global__ void __launch_bounds__(THREADS) binom5_kernel(const __grid_constant__
     if (__syncthreads_or(!mbar_wait_bounded(&sm.bar[0], 0, p.err))) return;
     const bool interior = interior5(p, x0, y0, 8 * R);
     if (!interior) {
-        fix_border5(sm.in[0].b, p, x0, y0, 8 * R + 4);
+        fix_border5(sm.in[0].b, p, x0, y0, 8 * R);
         __syncthreads();
     }
     binom5_tile<R>(sm.in[0].b, p, x0, y0, interior);
