@@ -343,9 +343,9 @@ hvx_status hvxQueryGraph(hvx_graph g, int32_t attribute, void* out, uint64_t siz
 /* Process n verified graphs in as few launches as possible on `stream`,
  * without waiting.  Graphs whose plans are one fused edge group (Gaussian3x3
  * -> Sobel3x3 -> Magnitude/Threshold and/or Phase) are run by one persistent
- * kernel over the tiles of all images, replayed from a captured CUDA graph
- * when the same set of graphs is submitted again; other graphs are run one
- * after another.  Image sizes may differ.  Wait with hvxWaitBatch. */
+ * kernel over the tiles of all images, tuned once per set of graphs; groups on
+ * one generated kernel or on the corner kernel share one launch as well; other
+ * graphs are run one after another.  Image sizes may differ.  Wait with hvxWaitBatch. */
 hvx_status hvxProcessGraphBatch(const hvx_graph* graphs, int32_t n, void* stream);
 hvx_status hvxWaitBatch(hvx_context ctx, void* stream);
 
@@ -356,8 +356,8 @@ hvx_status hvxWaitBatch(hvx_context ctx, void* stream);
  * tiles for that image (its tiles are 128 x 8R pixels; 0 where the batch runs
  * another kernel, which keeps its own tile), and *grid_out = the persistent
  * grid of its first launch (CTAs; 0 for a direct launch; a batch whose
- * size classes got different tile heights runs one launch per class, all
- * replayed from one captured CUDA graph).  rows_out holds n entries.
+ * size classes got different tile heights runs one launch per class).
+ * rows_out holds n entries.
  * HVX_ERROR_INVALID_PARAMETERS when no batch of these graphs has run since
  * they were last verified. */
 hvx_status hvxQueryBatch(const hvx_graph* graphs, int32_t n, int32_t* rows_out, int32_t* grid_out);

@@ -43,6 +43,15 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
+// launch_pdl, or a plain launch when the kernel must not begin early.
+template <class... KArgs, class... Args>
+cudaError_t launch_pdl_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                          cudaStream_t s, const Args&... args) {
+    if (early) return launch_pdl(kernel, grid, block, 0, s, args...);
+    kernel<<<grid, block, 0, s>>>(args...);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // TMA and mbarrier
 

@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(THREADS) binom5_batch_kernel(const EdgeBatchDe
             sm.ts[i] = __ldg(d.tile_start + i);
             if (i < d.n_img) sm.tx[i] = __ldg(d.tiles_x + i);
         }
+    pdl_wait();  // images only after the previous grid on the stream
     __syncthreads();
     if (threadIdx.x == 0)
         for (int s = 0; s < STAGES; ++s) {
@@ -277,6 +278,9 @@ __global__ void __launch_bounds__(THREADS) binom5_batch_kernel(const EdgeBatchDe
     bool failed = false;
     int k = 0;
     for (int t = first; t < d.total_tiles; t += gridDim.x, ++k) {
+        // The next launch may begin with this CTA's last tile (16 x 1920x1080: 19.2 us,
+        // 21.8 without overlap; 64: 57.1 and 60.2).
+        if (t + (int)gridDim.x >= d.total_tiles) pdl_launch_dependents();
         const int s = k % STAGES;
         const int ps = k % (STAGES + 1);
         const uint32_t parity = (uint32_t)(k / STAGES) & 1u;
@@ -320,12 +324,12 @@ cudaError_t launch_binom5(const CUtensorMap& map, const EdgeParams& p, cudaStrea
 }
 
 cudaError_t launch_binom5_batch(const EdgeBatchDesc& d, int grid, int rows, cudaStream_t s) {
+    const dim3 g(grid), b(THREADS);
     switch (rows) {
-        case 5: binom5_batch_kernel<5><<<grid, THREADS, 0, s>>>(d); break;
-        case 10: binom5_batch_kernel<10><<<grid, THREADS, 0, s>>>(d); break;
-        default: binom5_batch_kernel<MAXR><<<grid, THREADS, 0, s>>>(d); break;
+        case 5: return launch_pdl_if(d.early, binom5_batch_kernel<5>, g, b, s, d);
+        case 10: return launch_pdl_if(d.early, binom5_batch_kernel<10>, g, b, s, d);
+        default: return launch_pdl_if(d.early, binom5_batch_kernel<MAXR>, g, b, s, d);
     }
-    return cudaGetLastError();
 }
 
 int binom5_batch_blocks_per_sm() {

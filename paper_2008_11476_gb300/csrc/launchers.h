@@ -17,6 +17,8 @@ struct EdgeBatchDesc {
     int n_img;
     int total_tiles;
     int* err;
+    bool early;                  // the launch may begin before the stream's previous operation
+                                 // ends (maps, params and tables were in place before it)
 };
 
 // Output mode of an edge / Gaussian group (which kernel instantiation runs it);

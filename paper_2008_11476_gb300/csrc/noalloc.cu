@@ -183,6 +183,7 @@ extern "C" hvx_status hvxEdgeBatchNoAlloc(const hvx_edge_frame* frames, int32_t 
     d.n_img = n;
     d.total_tiles = tiles[n];
     d.err = d_err;
+    d.early = false;  // the tables are copied in on the same stream
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int per_sm = edge_batch_blocks_per_sm(edge_mode(params[0]));
