@@ -772,6 +772,7 @@ hvx_status hvxQueryGraph(hvx_graph hg, int32_t attr, void* out, uint64_t size) {
 hvx_status hvxProcessGraphBatch(const hvx_graph* gs, int32_t n, void* stream) {
     if (!gs || n <= 0) return HVX_ERROR_INVALID_PARAMETERS;
     std::vector<Graph*> v;
+    v.reserve((size_t)n);
     for (int i = 0; i < n; ++i) {
         if (!ok_graph(gs[i])) return HVX_ERROR_INVALID_REFERENCE;
         if (!G(gs[i])->verified) return HVX_ERROR_NOT_VERIFIED;
