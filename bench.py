@@ -5,7 +5,7 @@ Default workload (one JSON line on rank 0): the edge graph
 Gaussian3x3 -> Sobel3x3 -> Magnitude -> Threshold(100) + Phase on 1920x1080
 U8 frames (seeded rectangles + sigma-10 noise, BORDER_REPLICATE).  One step
 processes a batch of --frames frames resident in HBM with one persistent fused
-launch (hvxProcessGraphBatch, replayed from a captured CUDA graph).  The batch
+launch (hvxProcessGraphBatch, allowed to begin as the previous one ends).  The batch
 (--frames x 6.2 MB of external bytes) is larger than L2, so no flush is needed.
 
 The line reports: fused Mpix/s (value); the unfused one-launch-per-node form
@@ -880,8 +880,7 @@ def measure_harris(world, rank, local, torch, cpu, steps=5, warmup=3, codegen="a
 
 def measure_batch256(world, rank, local, torch, cpu, steps=10, warmup=3):
     """Config 4: 256 U8 images of seeded uneven sizes through the edge graph in
-    one persistent fused launch (replayed from a captured CUDA graph, grid
-    chosen by the autotuner); against one fused launch per image and 256
+    one persistent fused launch (grid chosen by the autotuner); against one fused launch per image and 256
     unfused runs of 5 launches each."""
     from paper_2008_11476_gb300 import graphs as PG
     from paper_2008_11476_gb300 import hvx as H
@@ -965,7 +964,7 @@ def measure_batch256(world, rank, local, torch, cpu, steps=10, warmup=3):
     unf = replica_mpix_s(mpix * 1e6, world, 3, tp)
     r = {"workload": "256 U8 images, w~U{320..3840}, h~U{240..2160} (seed 4; crops of seeded "
                      f"rectangles + noise frames), {mpix:.1f} Mpix per step, edge graph "
-                     "BORDER_REPLICATE, one persistent fused launch replayed from a CUDA graph",
+                     "BORDER_REPLICATE, one persistent fused launch",
          "value": round(value, 1), "unit": "Mpix/s", "ms_per_step": round(t / steps * 1e3, 4),
          "steps": steps,
          "roofline": hbm_roofline(3 * mpix * 1e6, t / steps, "edge_batch_kernel"),

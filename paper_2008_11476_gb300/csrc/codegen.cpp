@@ -1700,7 +1700,8 @@ bool set_maps(const JitKernel& k, HvxJitParams& p) {
 // measured points (FChain, Unsharp, Laplacian and a morphology graph; 64x48 to
 // 3840x2160; 1 to 16 frames; R = 3 .. 24): small launches want R = 3 (1080p
 // Unsharp frame: 5.0 us, 11.8 at R = 15), 16 x 1080p FChain R = 15 (57 us, 107
-// at R = 3), 16 x 1080p Unsharp R = 9 (25 us, 41 and 40 at R = 3 and 24).
+// at R = 3), 16 x 1080p Unsharp R = 9 (25 us, 41 and 40 at R = 3 and 24), all
+// before border tiles filled only the ring that is read (FChain now 52 us).
 // HVX_STRIP_ROWS in the environment overrides (0: the tile form).
 int strip_rows(const JitKernel& k, const int* W, const int* H, int n, int num_sms) {
     const int u = k.strip.unroll;

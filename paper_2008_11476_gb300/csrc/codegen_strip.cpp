@@ -12,10 +12,10 @@
 // operators are recomputed by each strip) or, for short groups, HBM.
 //
 // Measured against the tile form (GB300, one launch): FChain 16 x 1080p 126.5
-// -> 57 us (106 -> 35 instructions per pixel, issue 61 %), Unsharp 16 x
-// 2043x1361 77.7 -> 30.9 us (43 -> 11 instructions, 4.3 TB/s of reads and
-// writes), Laplacian 16 x 1080p 47.9 -> 24.3 us, a morphology graph on one
-// 1080p frame 18.8 -> 6.9 us, 64x48 frames equal.  Tried and left out:
+// -> 52 us (106 -> 35 instructions per pixel), Unsharp 16 x 2043x1361 77.8 ->
+// 26 us (43 -> 11 instructions, 5.1 TB/s of reads and writes), Laplacian 16 x
+// 1080p 47.9 -> 20.5 us, a morphology graph on one 1080p frame 18.7 -> 5.5 us,
+// 64x48 frames equal.  Tried and left out, at 61.7 and 37 us on the first two:
 // persistent CTAs with two box stages (FChain 65, Unsharp 48 us: the second
 // box costs more resident CTAs than the overlap gains back), one step
 // function with run-time stage conditions instead of the phases below (97 us:
