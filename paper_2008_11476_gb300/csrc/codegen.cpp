@@ -171,6 +171,7 @@ struct JitKernel {
     int smem_bytes = 0;
     int tw = 0, th = 0;
     std::vector<std::array<int, 3>> tma_boxes;  // tile form: (input, width, height)
+    bool read_only = false;  // tile form: reads images by read-only loads
     // the strip form (codegen_strip.cpp): compiled and run instead of the tile
     // form where the group has one
     bool strips = false;
@@ -241,6 +242,7 @@ struct Emitter {
     }
     bool tile_knobs = false;         // a tuning knob of the tile form is set: no strip form
     bool tma = true;                 // stage U8 inputs of interior tiles by TMA
+    bool read_only = false;          // some input is read by read-only loads
     std::vector<int> load_bar;       // per pass: word offset of its mbarrier, or -1
 
     static bool is_local(int op) {
@@ -865,7 +867,7 @@ struct Emitter {
     // unrolled so that they are all in flight at once.
     void emit_load(int b) {
         const int e = ext_in[b], h = d.buf[b].halo;
-        const std::string ld = "hvx_ld<" + std::to_string(d.in[e].fmt) + ">(p.in[" +
+        const std::string ld = "hvx_ld<" + std::to_string(d.in[e].fmt) + ", GMAP>(p.in[" +
                                std::to_string(e) + "], p.in_pitch[" + std::to_string(e) + "], ";
         o << "  // external input " << e << " -> B" << b << " (halo " << h << ")\n";
         if (tma_slot(b)) {  // interior tiles: the TMA box (emit_tma_load)
@@ -886,7 +888,10 @@ struct Emitter {
         }
         if (byte_slot(b)) {
             // interior tiles: the region's rows are inside the image, and the
-            // words [x0 - A, x0 + tw + A) stay inside each row's pitch
+            // words [x0 - A, x0 + tw + A) stay inside each row's pitch.  With
+            // HVX_CODEGEN_TMA=0 by read-only loads: such a kernel must not begin
+            // before the one ahead of it ends.
+            read_only = read_only || !tma;
             const int A = align_x(b), words = slot_w(b) / 4, rows = bh(b);
             o << "  if (!CHECK) {\n"
               << "    const unsigned char* const g0 = (const unsigned char*)p.in[" << e
@@ -896,9 +901,10 @@ struct Emitter {
               << "    for (int i = threadIdx.x; i < " << rows * words << "; i += " << kThreads
               << ") {\n"
               << "      const int r = i / " << words << ", k = i - r * " << words << ";\n"
-              << "      ((unsigned*)B" << b << ")[i] = __ldg((const unsigned*)(g0 + "
-                 "(unsigned long long)r * p.in_pitch["
-              << e << "]) + k);\n"
+              << "      ((unsigned*)B" << b << ")[i] = "
+              << (tma ? "(unsigned)hvx_ld<" + std::to_string(HVX_DF_S32) + ", GMAP>(g0, p.in_pitch["
+                      : std::string("__ldg((const unsigned*)(g0 + (unsigned long long)r * p.in_pitch["))
+              << e << (tma ? "], k, r);\n" : "]) + k);\n")
               << "    }\n  } else {\n";
             open_cells(bh(b), bw(b), h, h, true);
             o << "      int v;\n"
@@ -1169,7 +1175,7 @@ struct Emitter {
                 if (p.need_ld[b]) {
                     const int e = ext_in[b];
                     o << "        const int " << val(b) << " = in_img ? hvx_ld<" << d.in[e].fmt
-                      << ">(p.in[" << e << "], p.in_pitch[" << e << "], x, y) : 0;\n";
+                      << ", GMAP>(p.in[" << e << "], p.in_pitch[" << e << "], x, y) : 0;\n";
                 }
             for (int k = 0; k < d.n_stage; ++k) {
                 if (!p.need_op[k]) continue;
@@ -1384,15 +1390,28 @@ struct Emitter {
           << "  return m < n ? m : p - 1 - m;\n}\n"
           << "__device__ __forceinline__ int hvx_repeat(int v, int n) {\n"
           << "  const int m = v % n;\n  return m < 0 ? m + n : m;\n}\n"
-          << "template <int F>\n"
+          << "// Image loads are ordinary ones where the kernel before this one may write the\n"
+          << "// image while this one already runs (programmatic dependent launches): the\n"
+          << "// read-only path does not allow that.  RO: kernels launched in the ordinary way.\n"
+          << "template <int F, bool RO = false>\n"
           << "__device__ __forceinline__ int hvx_ld(const void* base, unsigned long long pitch, "
              "int x, int y) {\n"
           << "  const unsigned char* row = (const unsigned char*)base + (unsigned long long)y * "
              "pitch;\n"
-          << "  if (F == " << HVX_DF_U8 << ") return __ldg(row + x);\n"
-          << "  if (F == " << HVX_DF_S16 << ") return __ldg((const short*)row + x);\n"
-          << "  if (F == " << HVX_DF_UYVY << ") return __ldg((const unsigned short*)row + x);\n"
-          << "  return __ldg((const int*)row + x);\n}\n"
+          << "  if (RO) {\n"
+          << "    if (F == " << HVX_DF_U8 << ") return __ldg(row + x);\n"
+          << "    if (F == " << HVX_DF_S16 << ") return __ldg((const short*)row + x);\n"
+          << "    if (F == " << HVX_DF_UYVY << ") return __ldg((const unsigned short*)row + x);\n"
+          << "    return __ldg((const int*)row + x);\n  }\n"
+          << "  int v;\n"
+          << "  if (F == " << HVX_DF_U8
+          << ") asm volatile(\"ld.global.u8 %0, [%1];\" : \"=r\"(v) : \"l\"(row + x));\n"
+          << "  else if (F == " << HVX_DF_S16
+          << ") asm volatile(\"ld.global.s16 %0, [%1];\" : \"=r\"(v) : \"l\"(row + 2 * x));\n"
+          << "  else if (F == " << HVX_DF_UYVY
+          << ") asm volatile(\"ld.global.u16 %0, [%1];\" : \"=r\"(v) : \"l\"(row + 2 * x));\n"
+          << "  else asm volatile(\"ld.global.u32 %0, [%1];\" : \"=r\"(v) : \"l\"(row + 4 * x));\n"
+          << "  return v;\n}\n"
           << "template <int F>\n"
           << "__device__ __forceinline__ void hvx_st(void* base, unsigned long long pitch, int x, "
              "int y, int v) {\n"
@@ -1785,6 +1804,7 @@ JitKernel* find_kernel(const GenericDesc& d, const std::vector<std::string>& use
         slot->th = em.th;
         slot->smem_bytes = em.smem_words * 4;
         slot->tma_boxes = em.tma_boxes();
+        slot->read_only = em.read_only;
         slot->strips = strips;
         slot->strip = strip;
         slot->n_buf = d.n_buf;
@@ -1862,11 +1882,13 @@ bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code
 namespace {
 
 // A launch with programmatic stream serialisation: it may begin while the
-// previous kernel on the stream finishes (the kernel waits for it).
+// previous kernel on the stream finishes (the kernel waits for it).  early =
+// false: an ordinary one, for kernels whose read-only loads must not share
+// their lifetime with a kernel that writes the image.
 CUresult launch_dependent(CUfunction fn, unsigned gx, unsigned gy, unsigned gz, unsigned threads,
-                          int smem, cudaStream_t s, void** args) {
+                          int smem, cudaStream_t s, void** args, bool early = true) {
     const Driver& dr = driver();
-    if (!dr.launch_ex)
+    if (!dr.launch_ex || !early)
         return dr.launch(fn, gx, gy, gz, threads, 1, 1, (unsigned)smem, (CUstream)s, args, nullptr);
     CUlaunchAttribute attr = {};
     attr.id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
@@ -1890,7 +1912,7 @@ CUresult launch_dependent(CUfunction fn, unsigned gx, unsigned gy, unsigned gz, 
 cudaError_t jit_launch(const JitLaunch& j, cudaStream_t s) {
     void* args[] = {const_cast<HvxJitParams*>(&j.p)};
     return launch_dependent(j.k->fn, j.gx, j.gy, 1, j.p.rows ? STRIP_THREADS : kThreads, j.smem, s,
-                            args) == CUDA_SUCCESS
+                            args, j.p.rows || !j.k->read_only) == CUDA_SUCCESS
                ? cudaSuccess
                : cudaErrorLaunchFailure;
 }

@@ -26,6 +26,27 @@ __device__ __forceinline__ uint32_t byte_of(const uint4& v, int j) {
     return (w >> (8 * (j & 3))) & 0xFFu;
 }
 
+// Step i of an image's rows (per_row steps of 16 pixels each from column a0 on),
+// with its pixels where all 16 lie in columns v0 .. v2 - 1.  An ordinary load:
+// the kernel before this one may write the image while this one already runs
+// (programmatic dependent launches), which the read-only path does not allow.
+struct Step {
+    unsigned r;
+    int x;
+    bool full;
+    uint4 v;
+};
+__device__ __forceinline__ Step load_step(const uint8_t* base, uint64_t pitch, unsigned i,
+                                          unsigned per_row, int a0, int v0, int v2) {
+    Step s;
+    s.r = i / per_row;
+    s.x = a0 + 16 * (int)(i - s.r * per_row);
+    s.full = s.x >= v0 && s.x + 16 <= v2;
+    s.v = make_uint4(0u, 0u, 0u, 0u);
+    if (s.full) s.v = *reinterpret_cast<const uint4*>(base + (size_t)s.r * pitch + s.x);
+    return s;
+}
+
 __global__ void __launch_bounds__(kThreads) eqhist_count_kernel(const EqHistParams p) {
     __shared__ uint32_t bins[256 * kCopies];
     __shared__ uint32_t c[256];
@@ -39,18 +60,26 @@ __global__ void __launch_bounds__(kThreads) eqhist_count_kernel(const EqHistPara
     const int a0 = v0 & ~15, per_row = (v2 - a0 + 15) / 16;
     const unsigned copy = threadIdx.x & (kCopies - 1);
     const unsigned steps = v2 > v0 && h > 0 ? (unsigned)h * (unsigned)per_row : 0u;
-    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < steps; i += gridDim.x * kThreads) {
-        const unsigned r = i / (unsigned)per_row;
-        const int x = a0 + 16 * (int)(i - r * (unsigned)per_row);
-        const uint8_t* row = p.in + (size_t)(p.valid[1] + (int)r) * p.in_pitch;
-        if (x >= v0 && x + 16 <= v2) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + x));
+    const uint8_t* base = p.in + (size_t)p.valid[1] * p.in_pitch;
+    const unsigned stride = gridDim.x * kThreads;
+    unsigned i = blockIdx.x * kThreads + threadIdx.x;
+    Step s = {};
+    if (i < steps) s = load_step(base, p.in_pitch, i, (unsigned)per_row, a0, v0, v2);
+    while (i < steps) {
+        // the next step's load ahead of this one's atomics
+        Step n = {};
+        if (i + stride < steps)
+            n = load_step(base, p.in_pitch, i + stride, (unsigned)per_row, a0, v0, v2);
+        if (s.full) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) atomicAdd(&bins[byte_of(v, j) * kCopies + copy], 1u);
+            for (int j = 0; j < 16; ++j) atomicAdd(&bins[byte_of(s.v, j) * kCopies + copy], 1u);
         } else {
-            for (int j = max(x, v0); j < min(x + 16, v2); ++j)
+            const uint8_t* row = base + (size_t)s.r * p.in_pitch;
+            for (int j = max(s.x, v0); j < min(s.x + 16, v2); ++j)
                 atomicAdd(&bins[row[j] * kCopies + copy], 1u);
         }
+        s = n;
+        i += stride;
     }
     __syncthreads();
     const unsigned t = threadIdx.x;
@@ -98,32 +127,39 @@ __global__ void __launch_bounds__(kThreads) eqhist_map_kernel(const EqHistParams
     __shared__ uint8_t lut[256];
     pdl_launch_dependents();  // launched by launch_pdl
     pdl_wait();
-    lut[threadIdx.x] = __ldcg(p.lut + threadIdx.x);
+    lut[threadIdx.x] = p.lut[threadIdx.x];
     __syncthreads();
     const int W = (int)p.W, v0 = p.valid[0], v2 = p.valid[2];
-    const int per_row = (W + 15) / 16;
-    const unsigned steps = (unsigned)per_row * p.H;
-#pragma unroll 2
-    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < steps; i += gridDim.x * kThreads) {
-        const unsigned y = i / (unsigned)per_row;
-        const int x = 16 * (int)(i - y * (unsigned)per_row);
-        const uint8_t* in = p.in + (size_t)y * p.in_pitch;
-        uint8_t* out = p.out + (size_t)y * p.out_pitch;
-        const bool yin = (int)y >= p.valid[1] && (int)y < p.valid[3];
-        if (yin && x >= v0 && x + 16 <= v2) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(in + x));
-            uint32_t o[4];
+    const unsigned per_row = (unsigned)(W + 15) / 16, steps = per_row * p.H;
+    const unsigned stride = gridDim.x * kThreads;
+    for (unsigned i = blockIdx.x * kThreads + threadIdx.x; i < steps; i += 2 * stride) {
+        Step s[2];  // both loads ahead of the first store
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t lo = lut[byte_of(v, 4 * k)] | (uint32_t)lut[byte_of(v, 4 * k + 1)] << 8;
-                const uint32_t hi =
-                    lut[byte_of(v, 4 * k + 2)] | (uint32_t)lut[byte_of(v, 4 * k + 3)] << 8;
-                o[k] = lo | hi << 16;
+        for (int u = 0; u < 2; ++u)
+            if (i + u * stride < steps)
+                s[u] = load_step(p.in, p.in_pitch, i + u * stride, per_row, 0, v0, v2);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (i + u * stride >= steps) break;
+            const int x = s[u].x, y = (int)s[u].r;
+            uint8_t* out = p.out + (size_t)y * p.out_pitch;
+            const bool yin = y >= p.valid[1] && y < p.valid[3];
+            if (yin && s[u].full) {
+                uint32_t o[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t lo = lut[byte_of(s[u].v, 4 * k)] |
+                                        (uint32_t)lut[byte_of(s[u].v, 4 * k + 1)] << 8;
+                    const uint32_t hi = lut[byte_of(s[u].v, 4 * k + 2)] |
+                                        (uint32_t)lut[byte_of(s[u].v, 4 * k + 3)] << 8;
+                    o[k] = lo | hi << 16;
+                }
+                *reinterpret_cast<uint4*>(out + x) = make_uint4(o[0], o[1], o[2], o[3]);
+            } else {
+                const uint8_t* in = p.in + (size_t)y * p.in_pitch;
+                for (int j = x; j < min(x + 16, W); ++j)
+                    out[j] = yin && j >= v0 && j < v2 ? lut[in[j]] : 0;
             }
-            *reinterpret_cast<uint4*>(out + x) = make_uint4(o[0], o[1], o[2], o[3]);
-        } else {
-            for (int j = x; j < min(x + 16, W); ++j)
-                out[j] = yin && j >= v0 && j < v2 ? lut[in[j]] : 0;
         }
     }
 }
