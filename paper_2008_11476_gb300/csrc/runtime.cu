@@ -763,8 +763,9 @@ hvx_status check_device_error(Context* ctx) {
 }
 
 // Device result blocks of global operators (kept with the result image for
-// the life of the graph) and EqualizeHist's histogram.
-hvx_status alloc_results(Plan& P, Context* ctx) {
+// the life of the graph) and EqualizeHist's histogram; *clearing: a new block's
+// memset has been queued on the legacy stream.
+hvx_status alloc_result_blocks(Plan& P, Context* ctx, bool* clearing) {
     for (int i : P.order) {
         Op& op = P.ops[i];
         if (op_is_global(op.kind)) {
@@ -775,12 +776,20 @@ hvx_status alloc_results(Plan& P, Context* ctx) {
                 op.out->dev = nullptr;
             }
             if (!op.out->dev) {
-                hvx_status st = ctx->pool.alloc(n, &op.out->dev);
+                void* p = nullptr;
+                hvx_status st = ctx->pool.alloc(n, &p);
                 if (st != HVX_SUCCESS) return st;
+                cudaError_t e = cudaMemset(p, 0, n);
+                if (e == cudaSuccess) e = cudaMemset(p, global_result_fill(op.kind), res);
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    ctx->pool.free(p);
+                    return cuda_status(e);
+                }
+                op.out->dev = p;
                 op.out->owns_mem = true;
                 op.out->bytes = n;
-                cudaMemset(op.out->dev, 0, n);
-                cudaMemset(op.out->dev, global_result_fill(op.kind), res);
+                *clearing = true;
             }
             if (!op.out->mirror && ctx->host.alloc(res, &op.out->mirror, &op.out->mirror_dev)) {
                 op.out->mirror_bytes = res;
@@ -788,14 +797,34 @@ hvx_status alloc_results(Plan& P, Context* ctx) {
             }
         }
         if (op.kind == OP_EQHIST && !op.node->d_aux) {
-            if (cudaMalloc(&op.node->d_aux, EQHIST_BYTES) != cudaSuccess) {
+            void* p = nullptr;
+            if (cudaMalloc(&p, EQHIST_BYTES) != cudaSuccess) {
                 cudaGetLastError();
                 return HVX_ERROR_NO_MEMORY;
             }
-            cudaMemset(op.node->d_aux, 0, EQHIST_BYTES);
+            const cudaError_t e = cudaMemset(p, 0, EQHIST_BYTES);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                cudaFree(p);
+                return cuda_status(e);
+            }
+            op.node->d_aux = p;
+            *clearing = true;
         }
     }
     return HVX_SUCCESS;
+}
+
+// The blocks, cleared on return: kernels only restore the scratch in them, and
+// the graph may first run on a stream that does not wait for the legacy one.
+hvx_status alloc_results(Plan& P, Context* ctx) {
+    bool clearing = false;
+    hvx_status st = alloc_result_blocks(P, ctx, &clearing);
+    if (clearing) {
+        const cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+        if (st == HVX_SUCCESS) st = cuda_status(e);
+    }
+    return st;
 }
 
 hvx_status prepare_launches(Graph* g) {
