@@ -297,7 +297,13 @@ hvx_status hvxProcessGraph(hvx_graph g);
 
 /* Enqueue a verified graph on `stream` and return without waiting.
  * hvxWaitGraph waits for the last scheduled run and reports a device-side
- * error (HVX_ERROR_TIMEOUT if a kernel's bounded wait ran out). */
+ * error (HVX_ERROR_TIMEOUT if a kernel's bounded wait ran out).
+ *
+ * Runs of one graph that has MeanStdDev, MinMaxLoc, Histogram or EqualizeHist
+ * nodes never overlap (each starts from state that the one before left on the
+ * device): a run on another stream than the graph's previous one waits for
+ * that one, also in batches and on servers.  Stream captures are outside this:
+ * replays of such a graph must not overlap its other runs. */
 hvx_status hvxScheduleGraph(hvx_graph g, void* stream);
 hvx_status hvxWaitGraph(hvx_graph g);
 
@@ -345,7 +351,9 @@ hvx_status hvxQueryGraph(hvx_graph g, int32_t attribute, void* out, uint64_t siz
  * -> Sobel3x3 -> Magnitude/Threshold and/or Phase) are run by one persistent
  * kernel over the tiles of all images, tuned once per set of graphs; groups on
  * one generated kernel or on the corner kernel share one launch as well; other
- * graphs are run one after another.  Image sizes may differ.  Wait with hvxWaitBatch. */
+ * graphs are run one after another, and so is a batch in which a graph with
+ * MeanStdDev, MinMaxLoc, Histogram or EqualizeHist nodes occurs more than once.
+ * Image sizes may differ.  Wait with hvxWaitBatch. */
 hvx_status hvxProcessGraphBatch(const hvx_graph* graphs, int32_t n, void* stream);
 hvx_status hvxWaitBatch(hvx_context ctx, void* stream);
 

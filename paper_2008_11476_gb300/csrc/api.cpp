@@ -137,6 +137,7 @@ void maybe_destroy(Image* im) {
 
 void destroy_graph(Graph* g) {
     if (g->scheduled && g->done) cudaEventSynchronize(g->done);
+    if (g->ordered) cudaEventSynchronize(g->order);  // (its blocks go to other graphs)
     release_plan(g);
     for (auto& n : g->nodes) {
         if (n->d_aux) cudaFree(n->d_aux);
@@ -151,6 +152,7 @@ void destroy_graph(Graph* g) {
     for (Image* v : g->virtuals) destroy_image(v);
     g->virtuals.clear();
     if (g->done) cudaEventDestroy(g->done);
+    if (g->order) cudaEventDestroy(g->order);
     g->magic = 0;
     Context* ctx = g->ctx;
     auto& gv = ctx->graphs;

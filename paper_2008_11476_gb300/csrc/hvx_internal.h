@@ -279,6 +279,10 @@ struct Plan {
     uint64_t intermediate_bytes = 0;
     uint64_t external_bytes = 0;
     std::string kernel_kinds;
+    // Launches leave state in device memory that the next one starts from
+    // (results of global operators and their scratch, EqualizeHist's bins):
+    // they never overlap.
+    bool stateful = false;
 };
 
 struct Graph {
@@ -296,6 +300,11 @@ struct Graph {
     bool scheduled = false;
     bool settled = false;        // nothing launched since the last wait for the graph
     cudaStream_t last_stream = nullptr;
+    // stateful plans: recorded after every launch, which the next one waits for
+    // on another stream
+    cudaEvent_t order = nullptr;
+    cudaStream_t order_stream = nullptr;
+    bool ordered = false;
     std::atomic<int> busy{0};  // in flight on a server
 };
 

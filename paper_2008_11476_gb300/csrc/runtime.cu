@@ -838,6 +838,9 @@ hvx_status prepare_launches(Graph* g) {
     // HVX_CODEGEN_ONLY: generated kernels in place of the hand-written ones
     const bool hand = g->codegen != HVX_CODEGEN_ONLY;
     const bool must_gen = g->codegen == HVX_CODEGEN_REQUIRE || g->codegen == HVX_CODEGEN_ONLY;
+    P.stateful = false;
+    for (int i : P.order)
+        P.stateful = P.stateful || op_is_global(P.ops[i].kind) || P.ops[i].kind == OP_EQHIST;
     for (Group& G : P.groups) {
         G.ext_bytes = G.mem_bytes = 0;
         for (Image* im : G.inputs) {
@@ -916,10 +919,40 @@ hvx_status prepare_launches(Graph* g) {
     return HVX_SUCCESS;
 }
 
-hvx_status launch_plan(Graph* g, cudaStream_t s) {
-    if (fault_fires(HVX_FAULT_LAUNCH)) return HVX_ERROR_DEVICE;  // injected, nothing enqueued
-    bind_device(g->ctx);
-    g->settled = false;
+namespace {
+
+// Before a launch of g on s: behind g's previous launch when that ran on another
+// stream (two threads' per-thread streams share a handle).  *track: note_launch
+// follows.  Under stream capture neither happens: the order of replays is the
+// caller's (hvx.h).
+hvx_status order_launch(Graph* g, cudaStream_t s, bool* track) {
+    *track = false;
+    if (!g->plan.stateful) return HVX_SUCCESS;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cs);
+    if (e == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+        *track = true;
+        if (g->ordered && (s != g->order_stream || s == cudaStreamPerThread))
+            e = cudaStreamWaitEvent(s, g->order, 0);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return cuda_status(e);
+}
+
+hvx_status note_launch(Graph* g, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (!g->order) e = cudaEventCreateWithFlags(&g->order, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(g->order, s);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return cuda_status(e);
+    }
+    g->order_stream = s;
+    g->ordered = true;
+    return HVX_SUCCESS;
+}
+
+hvx_status launch_groups(Graph* g, cudaStream_t s) {
     for (Group& G : g->plan.groups) {
         NvtxRange nvtx(G.jit_on ? "hvx launch generated" : group_kernel_name(G.kernel));
         cudaError_t e = cudaSuccess;
@@ -940,6 +973,23 @@ hvx_status launch_plan(Graph* g, cudaStream_t s) {
         if (e != cudaSuccess) return cuda_status(e);
     }
     return HVX_SUCCESS;
+}
+
+}  // namespace
+
+hvx_status launch_plan(Graph* g, cudaStream_t s) {
+    if (fault_fires(HVX_FAULT_LAUNCH)) return HVX_ERROR_DEVICE;  // injected, nothing enqueued
+    bind_device(g->ctx);
+    g->settled = false;
+    bool track = false;
+    hvx_status st = order_launch(g, s, &track);
+    if (st != HVX_SUCCESS) return st;
+    st = launch_groups(g, s);
+    if (track) {  // (also behind the groups that were launched before an error)
+        const hvx_status noted = note_launch(g, s);
+        if (st == HVX_SUCCESS) st = noted;
+    }
+    return st;
 }
 
 // ---------------------------------------------------------------------------
@@ -1417,6 +1467,12 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
                        P.groups[0].jit_on && (!jk || P.groups[0].jit.k == jk);
             if (jit_same) jk = P.groups[0].jit.k;
         }
+        // (a graph with state that occurs twice runs twice, one after the other)
+        if (jit_same && gs[0]->plan.stateful) {
+            std::vector<Graph*> sorted(gs, gs + n);
+            std::sort(sorted.begin(), sorted.end());
+            jit_same = std::adjacent_find(sorted.begin(), sorted.end()) == sorted.end();
+        }
         // one launch when every plan is a single corner group on the strip kernel
         // with the same response (Harris or Shi-Tomasi)
         bool harris_same = !jit_same;
@@ -1467,15 +1523,23 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
     }
     hit->last_use = ++bc->tick;
     if (hit->jit.k) {
+        // (one kernel: all of the graphs have state, or none)
+        bool track = false;
+        for (int i = 0; i < n && gs[0]->plan.stateful; ++i) {
+            const hvx_status st = order_launch(gs[i], s, &track);
+            if (st != HVX_SUCCESS) return st;
+        }
         for (int i = 0; i < n; ++i)
             for (const ResultReset& rr : gs[i]->plan.groups[0].resets) {
                 cudaError_t e = cudaMemsetAsync(rr.p, rr.byte, rr.n, s);
                 if (e != cudaSuccess) return cuda_status(e);
             }
         const uint8_t* base = static_cast<const uint8_t*>(hit->dmem);
-        return cuda_status(jit_launch_batch(
+        hvx_status st = cuda_status(jit_launch_batch(
             hit->jit, reinterpret_cast<const HvxJitParams*>(base),
             reinterpret_cast<const int*>(base + (size_t)n * sizeof(HvxJitParams)), s));
+        for (int i = 0; i < n && track && st == HVX_SUCCESS; ++i) st = note_launch(gs[i], s);
+        return st;
     }
     if (hit->harris) {
         const uint8_t* base = static_cast<const uint8_t*>(hit->dmem);

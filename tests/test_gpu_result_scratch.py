@@ -71,3 +71,77 @@ def test_first_launch_on_a_stream_that_does_not_wait(ctx, w, h):
     H.hvxScheduleGraph(s.g, side.cuda_stream)
     H.hvxWaitGraph(s.g)
     s.check()
+
+
+def single_group(ctx, w, h, seed, codegen=H.HVX_CODEGEN_AUTO):
+    """MeanStdDev, MinMaxLoc and Histogram of a Dilate3x3 in one launch."""
+    img = synth.rects_noise(w, h, seed)
+    g = H.hvxCreateGraph(ctx)
+    d = H.hvxCreateVirtualImage(g)
+    H.hvxDilate3x3Node(g, PG.upload(ctx, img, H.HVX_DF_U8), d)
+    nodes = (H.hvxMeanStdDevNode(g, d), H.hvxMinMaxLocNode(g, d),
+             H.hvxHistogramNode(g, d, 256, 0, 256))
+    H.hvxSetGraphCodegen(g, codegen)
+    H.hvxVerifyGraph(g)
+    assert H.hvxQueryGraph(g, H.HVX_GRAPH_NUM_LAUNCHES) == 1
+    return g, nodes, O.morph3x3(img, O.MORPH_DILATE)
+
+
+def check_group(nodes, ref):
+    m = H.hvxGetNodeResult(nodes[0], H.HvxMeanStdDev())
+    assert (m.sum, m.sum_squares, m.count) == O.mean_stddev(ref)[2]
+    r, want = H.hvxGetNodeResult(nodes[1], H.HvxMinMaxLoc()), O.minmaxloc(ref)
+    assert (r.min, r.max, r.min_count, r.max_count) == (want["min"], want["max"],
+                                                        want["min_count"], want["max_count"])
+    np.testing.assert_array_equal(H.hvxGetNodeResult(nodes[2], np.zeros(256, np.uint32)),
+                                  O.histogram(ref, 256, 0, 256))
+
+
+@pytest.mark.parametrize("codegen", [H.HVX_CODEGEN_OFF, H.HVX_CODEGEN_REQUIRE])
+def test_graph_that_occurs_twice_in_a_batch(ctx, codegen):
+    graphs = [single_group(ctx, w, h, w, codegen) for w, h in [(640, 480), (7, 5), (1920, 1080)]]
+    for order in ([0, 2, 0, 1, 2, 2], [0, 1, 2], [2, 2], [1]):
+        for _ in range(2):
+            H.hvxProcessGraphBatch([graphs[i][0] for i in order])
+            H.hvxWaitBatch(ctx)
+            for i in order:
+                check_group(*graphs[i][1:])
+
+
+def test_graph_on_several_streams_without_waits(ctx):
+    s = Statistics(ctx, 1920, 1080, seed=8)
+    H.hvxVerifyGraph(s.g)
+    g, nodes, ref = single_group(ctx, 1921, 1081, 9)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    for k in range(30):
+        H.hvxScheduleGraph(s.g, streams[k % 3].cuda_stream)
+        # alone and as a batch in turn
+        if k % 2:
+            H.hvxProcessGraphBatch([g], streams[(k + 1) % 3].cuda_stream)
+        else:
+            H.hvxScheduleGraph(g, streams[(k + 2) % 3].cuda_stream)
+    torch.cuda.synchronize()
+    s.check()
+    check_group(nodes, ref)
+    # a server between two runs on a stream
+    server = H.hvxCreateServer(ctx, 0, 4, 4)
+    for _ in range(5):
+        H.hvxScheduleGraph(s.g, streams[0].cuda_stream)
+        ticket = H.hvxServerSubmit(server, s.g)
+        H.hvxServerWait(server, ticket)
+        s.check()
+    H.hvxReleaseServer(server)
+
+
+def test_blocks_of_a_released_graph_are_idle(ctx):
+    """A graph released right after its launch: its blocks go to a new graph of
+    the same shape, whose first run must find them clear."""
+    side = torch.cuda.Stream()
+    for k in range(10):
+        g, _, _ = single_group(ctx, 1920, 1080, k)
+        H.hvxProcessGraphBatch([g], side.cuda_stream)
+        H.hvxReleaseGraph(g)
+        g, nodes, ref = single_group(ctx, 640, 480, 20 + k)
+        H.hvxProcessGraph(g)
+        check_group(nodes, ref)
+        H.hvxReleaseGraph(g)
