@@ -353,7 +353,12 @@ hvx_status hvxQueryGraph(hvx_graph g, int32_t attribute, void* out, uint64_t siz
  * one generated kernel or on the corner kernel share one launch as well; other
  * graphs are run one after another, and so is a batch in which a graph with
  * MeanStdDev, MinMaxLoc, Histogram or EqualizeHist nodes occurs more than once.
- * Image sizes may differ.  Wait with hvxWaitBatch. */
+ * Image sizes may differ.  Wait with hvxWaitBatch.
+ *
+ * On a stream that is being captured, batches on one generated kernel or on the
+ * corner kernel are captured, and the context keeps their tables until it is
+ * released; batches of edge, Gaussian3x3 or 5x5 binomial graphs are refused
+ * (HVX_ERROR_DEVICE) and leave the capture as it is. */
 hvx_status hvxProcessGraphBatch(const hvx_graph* graphs, int32_t n, void* stream);
 hvx_status hvxWaitBatch(hvx_context ctx, void* stream);
 

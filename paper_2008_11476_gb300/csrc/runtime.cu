@@ -1009,6 +1009,7 @@ struct BatchEntry {
     std::vector<EdgeLaunch> edge;  // edge / Gaussian batch: its launches
     int edge_mode = 0;
     uint64_t last_use = 0;
+    bool captured = false;  // a stream capture holds its tables: never evicted
     int grid = 0;  // persistent CTAs chosen by the autotuner
     // generated-kernel batches: one direct launch over every image's tiles
     JitBatch jit;
@@ -1022,17 +1023,25 @@ struct BatchEntry {
     std::vector<void*> more_dmem;  // edge batch split by size class: the other tables
 };
 
-// A batch's tables to the device, complete on return (its launches read them
-// without waiting for the stream's previous work, on any stream).
-cudaError_t upload(void* dev, const void* host, size_t bytes) {
-    const cudaError_t e = cudaMemcpy(dev, host, bytes, cudaMemcpyHostToDevice);
-    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
-}
-
 struct BatchCache {
     std::vector<BatchEntry> entries;
-    cudaStream_t trial = nullptr;  // the autotuner's launches
+    cudaStream_t trial = nullptr;  // the autotuner's launches, uploads of tables
     uint64_t tick = 0;
+};
+
+// A batch's tables to the device, complete on return (its launches read them
+// without waiting for the stream's previous work, on any stream).  By the
+// internal stream: the legacy one is closed while a blocking stream is captured.
+cudaError_t upload(BatchCache* bc, void* dev, const void* host, size_t bytes) {
+    const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, bc->trial);
+    return e == cudaSuccess ? cudaStreamSynchronize(bc->trial) : e;
+}
+
+// While it lives, the thread may allocate although a stream is being captured.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
 void destroy_batch_cache(Context* ctx) {
@@ -1107,7 +1116,7 @@ int autotune_grid(Context* ctx, BatchCache* bc, const EdgeBatchDesc& d, int mode
 // parameter block and its tile counts, for `rows` rows per thread (edge
 // modes: tiles of 128 x 8R and boxes of 160 x (8R + 4); the Gaussian kernel
 // keeps its own tile).  One device block; *d describes it.
-hvx_status make_edge_tables(Context* ctx, Graph* const* gs, int n, int mode, int rows,
+hvx_status make_edge_tables(Context* ctx, BatchCache* bc, Graph* const* gs, int n, int mode, int rows,
                             void** dmem_out, EdgeBatchDesc* d) {
     const size_t maps_bytes = (size_t)n * sizeof(CUtensorMap);
     const size_t params_off = maps_bytes;
@@ -1148,7 +1157,7 @@ hvx_status make_edge_tables(Context* ctx, Graph* const* gs, int n, int mode, int
         cudaGetLastError();
         return HVX_ERROR_NO_MEMORY;
     }
-    e = upload(dmem, host.data(), total);
+    e = upload(bc, dmem, host.data(), total);
     if (e != cudaSuccess) {
         cudaFree(dmem);
         return cuda_status(e);
@@ -1204,11 +1213,6 @@ float time_launches(BatchCache* bc, const std::vector<EdgeLaunch>& ls, int mode)
 // 15) gives every image 128 x 8R tiles in a single launch, without trials.
 hvx_status build_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int n, int mode,
                              cudaStream_t user_stream, BatchEntry& out) {
-    cudaError_t e;
-    if (!bc->trial) {
-        e = cudaStreamCreateWithFlags(&bc->trial, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return cuda_status(e);
-    }
     const int grid_max = ctx->num_sms * std::max(1, edge_batch_blocks_per_sm(mode));
     std::vector<void*> blocks;
     auto release = [&] {
@@ -1225,7 +1229,7 @@ hvx_status build_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int
             EdgeLaunch l;
             l.rows = rows[k];
             void* dm = nullptr;
-            hvx_status st = make_edge_tables(ctx, sub.data(), (int)sub.size(), mode, l.rows, &dm,
+            hvx_status st = make_edge_tables(ctx, bc, sub.data(), (int)sub.size(), mode, l.rows, &dm,
                                              &l.d);
             if (st != HVX_SUCCESS) return st;
             blocks.push_back(dm);
@@ -1324,7 +1328,8 @@ hvx_status build_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int
 // Batch of graphs whose plans are one group running the same generated
 // kernel: the images' launch parameters and tile prefix sums in one device
 // block.
-hvx_status build_jit_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEntry& out) {
+hvx_status build_jit_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int n,
+                                 BatchEntry& out) {
     std::vector<const JitLaunch*> js(n);
     for (int i = 0; i < n; ++i) js[i] = &gs[i]->plan.groups[0].jit;
     std::vector<HvxJitParams> ps(n);
@@ -1344,7 +1349,7 @@ hvx_status build_jit_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEnt
         cudaGetLastError();
         return HVX_ERROR_NO_MEMORY;
     }
-    e = upload(dmem, host.data(), total);
+    e = upload(bc, dmem, host.data(), total);
     if (e != cudaSuccess) {
         cudaFree(dmem);
         return cuda_status(e);
@@ -1359,7 +1364,8 @@ hvx_status build_jit_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEnt
 // Batch of corner graphs on the strip kernel: one rows-per-thread for all of
 // them, each input's tensor map boxed for it, then maps, parameters and tile
 // tables in one device block.
-hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, BatchEntry& out) {
+hvx_status build_harris_batch_entry(Context* ctx, BatchCache* bc, Graph* const* gs, int n,
+                                    BatchEntry& out) {
     std::vector<int> ws(n), hs(n);
     for (int i = 0; i < n; ++i) {
         ws[i] = (int)gs[i]->plan.groups[0].W;
@@ -1399,7 +1405,7 @@ hvx_status build_harris_batch_entry(Context* ctx, Graph* const* gs, int n, Batch
         cudaGetLastError();
         return HVX_ERROR_NO_MEMORY;
     }
-    e = upload(dmem, host.data(), total);
+    e = upload(bc, dmem, host.data(), total);
     if (e != cudaSuccess) {
         cudaFree(dmem);
         return cuda_status(e);
@@ -1445,6 +1451,16 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
     // a batch seen before, by graph and plan: nothing of it is looked at again
     if (!ctx->batch) ctx->batch = new BatchCache();
     BatchCache* bc = ctx->batch;
+    // Under the caller's stream capture generated and corner batches are captured,
+    // and keep their tables until the context is released; edge, Gaussian and
+    // binomial batches are refused, before anything would disturb the capture.
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t ce = cudaStreamIsCapturing(s, &cs);
+    if (ce != cudaSuccess) {
+        cudaGetLastError();
+        return cuda_status(ce);
+    }
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
     BatchEntry* hit = nullptr;
     for (BatchEntry& e : bc->entries) {
         if ((int)e.graphs.size() != n) continue;
@@ -1504,24 +1520,37 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             }
             return HVX_SUCCESS;
         }
-        if (bc->entries.size() >= 16) {
-            auto oldest = std::min_element(
-                bc->entries.begin(), bc->entries.end(),
-                [](const BatchEntry& a, const BatchEntry& b) { return a.last_use < b.last_use; });
+        if (capturing && same) return cuda_status(cudaErrorStreamCaptureUnsupported);
+        // the least recently used of 16 or more batches makes room (by a wait for
+        // the stream and a free: not while it is captured)
+        auto oldest = bc->entries.end();
+        for (auto e = bc->entries.begin(); e != bc->entries.end(); ++e)
+            if (!e->captured && (oldest == bc->entries.end() || e->last_use < oldest->last_use))
+                oldest = e;
+        const auto free_use = std::count_if(bc->entries.begin(), bc->entries.end(),
+                                            [](const BatchEntry& e) { return !e.captured; });
+        if (free_use >= 16 && !capturing) {
             cudaStreamSynchronize(s);
             if (oldest->dmem) cudaFree(oldest->dmem);
             for (void* p : oldest->more_dmem) cudaFree(p);
             bc->entries.erase(oldest);
         }
+        RelaxedCapture relaxed;
+        if (!bc->trial) {
+            const cudaError_t e = cudaStreamCreateWithFlags(&bc->trial, cudaStreamNonBlocking);
+            if (e != cudaSuccess) return cuda_status(e);
+        }
         BatchEntry fresh;
-        hvx_status st = jit_same      ? build_jit_batch_entry(ctx, gs, n, fresh)
-                        : harris_same ? build_harris_batch_entry(ctx, gs, n, fresh)
+        hvx_status st = jit_same      ? build_jit_batch_entry(ctx, bc, gs, n, fresh)
+                        : harris_same ? build_harris_batch_entry(ctx, bc, gs, n, fresh)
                                       : build_batch_entry(ctx, bc, gs, n, mode, s, fresh);
         if (st != HVX_SUCCESS) return st;
         bc->entries.push_back(fresh);
         hit = &bc->entries.back();
     }
+    if (capturing && !hit->edge.empty()) return cuda_status(cudaErrorStreamCaptureUnsupported);
     hit->last_use = ++bc->tick;
+    hit->captured = hit->captured || capturing;
     if (hit->jit.k) {
         // (one kernel: all of the graphs have state, or none)
         bool track = false;
@@ -1555,13 +1584,7 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
     }
     // Direct launches that may begin while the previous one ends (replaying a
     // captured graph instead: 8.3 against 4.0 us for 4 Gaussians of 640x480, 53.6
-    // against 35.9 us for 16 of 2043x1361).  Not under the caller's stream capture:
-    // the tables live only until 16 other batches have run.
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaError_t ce = cudaStreamIsCapturing(s, &cs);
-    if (ce == cudaSuccess && cs != cudaStreamCaptureStatusNone)
-        ce = cudaErrorStreamCaptureUnsupported;
-    if (ce != cudaSuccess) return cuda_status(ce);
+    // against 35.9 us for 16 of 2043x1361).
     for (const EdgeLaunch& l : hit->edge) {
         const cudaError_t e = launch_edge_batch(l.d, hit->edge_mode, l.grid, s, l.rows);
         if (e != cudaSuccess) return cuda_status(e);
