@@ -667,6 +667,7 @@ hvx_status hvxScheduleGraph(hvx_graph hg, void* stream) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     hvx_status st = launch_plan(g, s);
     if (st != HVX_SUCCESS) return set_last(g, st);
+    g->done_launch = g->launches;
     if (cudaEventRecord(g->done, s) != cudaSuccess) {
         cudaGetLastError();
         return set_last(g, HVX_ERROR_DEVICE);
@@ -683,7 +684,7 @@ hvx_status hvxWaitGraph(hvx_graph hg) {
     cudaError_t e = cudaEventSynchronize(g->done);
     g->scheduled = false;
     if (e != cudaSuccess) return set_last(g, cuda_status(e));
-    g->settled = true;
+    g->settled = g->done_launch == g->launches && !g->captured;
     return set_last(g, check_device_error(g->ctx));
 }
 
@@ -1143,7 +1144,7 @@ hvx_status hvxGetNodeResult(hvx_node hn, void* out, uint64_t size) {
     if (n->graph->ctx->plan_only) return HVX_ERROR_NOT_SUPPORTED;
     Image* r = n->out[0];
     if (!r || !r->dev) return HVX_ERROR_NOT_VERIFIED;
-    // the host's copy where the plan writes one: no copy, and no wait when the
+    // the host's copy where the last launch wrote it: no copy, and no wait when the
     // graph has been waited for (else for the default stream's work, as a
     // synchronous copy does)
     auto fetch = [&](void* to, uint64_t bytes) {

@@ -111,7 +111,7 @@ struct Image {
     // holds the device result block.
     bool is_result = false;
     // A result's copy in host memory that the device writes (HostBlock), and
-    // whether the graph's plan writes it.
+    // whether the last launch wrote it (else dev alone).
     void* mirror = nullptr;
     void* mirror_dev = nullptr;
     uint64_t mirror_bytes = 0;
@@ -265,6 +265,8 @@ struct Group {
     bool jit_on = false;
     EqHistParams eqh;            // GK_EQHIST
     std::vector<ResultReset> resets;
+    std::vector<Image*> results;  // of its global operators
+    bool mirrored = false;        // its launches write the results' host copies
     std::vector<std::string> user_code;  // user-defined operators' code (GenStage.i0)
     uint64_t ext_bytes = 0;      // bytes of non-virtual images read + written
     uint64_t mem_bytes = 0;      // bytes of every image read + written
@@ -298,7 +300,11 @@ struct Graph {
     Plan plan;
     cudaEvent_t done = nullptr;
     bool scheduled = false;
-    bool settled = false;        // nothing launched since the last wait for the graph
+    // launches so far, and the one that `done` was recorded behind; settled: no
+    // launch since the last wait for the graph
+    uint64_t launches = 0, done_launch = 0;
+    bool settled = false;
+    bool captured = false;  // a stream capture may launch it at any time
     cudaStream_t last_stream = nullptr;
     // stateful plans: recorded after every launch, which the next one waits for
     // on another stream

@@ -856,8 +856,11 @@ hvx_status prepare_launches(Graph* g) {
         HarrisMatch hm;
         const Op& first = P.ops[G.ops[0]];
         G.resets.clear();
+        G.results.clear();
+        G.mirrored = false;
         for (int i : G.ops) {
             const Op& op = P.ops[i];
+            if (op_is_global(op.kind)) G.results.push_back(op.out);
             if (op_is_global(op.kind) && op.out->dev)
                 G.resets.push_back({op.out->dev, global_result_fill(op.kind),
                                     global_result_bytes(op.kind, op.node->p.hist_bins)});
@@ -902,11 +905,8 @@ hvx_status prepare_launches(Graph* g) {
                                        &why);
                 G.jit.p.err = ctx->d_error;
                 // the strip form's last CTA writes the whole result, and its mirror
-                const bool strips = G.jit_on && G.jit.p.rows > 0;
-                if (strips) G.resets.clear();
-                for (int i : G.ops)
-                    if (op_is_global(P.ops[i].kind))
-                        P.ops[i].out->mirror_live = strips && P.ops[i].out->mirror;
+                G.mirrored = G.jit_on && G.jit.p.rows > 0;
+                if (G.mirrored) G.resets.clear();
                 if (!G.jit_on && getenv("HVX_CODEGEN_VERBOSE"))
                     fprintf(stderr, "hvx: no generated kernel for a group: %s\n", why.c_str());
                 if (!G.jit_on && (must_gen || user))
@@ -934,6 +934,8 @@ hvx_status order_launch(Graph* g, cudaStream_t s, bool* track) {
         *track = true;
         if (g->ordered && (s != g->order_stream || s == cudaStreamPerThread))
             e = cudaStreamWaitEvent(s, g->order, 0);
+    } else {
+        g->captured = true;
     }
     if (e != cudaSuccess) cudaGetLastError();
     return cuda_status(e);
@@ -950,6 +952,11 @@ hvx_status note_launch(Graph* g, cudaStream_t s) {
     g->order_stream = s;
     g->ordered = true;
     return HVX_SUCCESS;
+}
+
+// A group has been launched: where its results will be.
+void note_results(Group& G) {
+    for (Image* r : G.results) r->mirror_live = G.mirrored && r->mirror;
 }
 
 hvx_status launch_groups(Graph* g, cudaStream_t s) {
@@ -971,6 +978,7 @@ hvx_status launch_groups(Graph* g, cudaStream_t s) {
             default: e = G.jit_on ? jit_launch(G.jit, s) : launch_generic(G.gdesc, s); break;
         }
         if (e != cudaSuccess) return cuda_status(e);
+        note_results(G);
     }
     return HVX_SUCCESS;
 }
@@ -980,6 +988,7 @@ hvx_status launch_groups(Graph* g, cudaStream_t s) {
 hvx_status launch_plan(Graph* g, cudaStream_t s) {
     if (fault_fires(HVX_FAULT_LAUNCH)) return HVX_ERROR_DEVICE;  // injected, nothing enqueued
     bind_device(g->ctx);
+    ++g->launches;
     g->settled = false;
     bool track = false;
     hvx_status st = order_launch(g, s, &track);
@@ -1447,7 +1456,10 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
     NvtxRange nvtx("hvx batch");
     std::lock_guard<std::mutex> lock(ctx->batch_mu);
     bind_device(ctx);
-    for (int i = 0; i < n; ++i) gs[i]->settled = false;
+    for (int i = 0; i < n; ++i) {
+        ++gs[i]->launches;
+        gs[i]->settled = false;
+    }
     // a batch seen before, by graph and plan: nothing of it is looked at again
     if (!ctx->batch) ctx->batch = new BatchCache();
     BatchCache* bc = ctx->batch;
@@ -1567,7 +1579,10 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
         hvx_status st = cuda_status(jit_launch_batch(
             hit->jit, reinterpret_cast<const HvxJitParams*>(base),
             reinterpret_cast<const int*>(base + (size_t)n * sizeof(HvxJitParams)), s));
-        for (int i = 0; i < n && track && st == HVX_SUCCESS; ++i) st = note_launch(gs[i], s);
+        for (int i = 0; i < n && st == HVX_SUCCESS; ++i) {
+            note_results(gs[i]->plan.groups[0]);
+            if (track) st = note_launch(gs[i], s);
+        }
         return st;
     }
     if (hit->harris) {
