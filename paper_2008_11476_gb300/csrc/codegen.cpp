@@ -178,10 +178,12 @@ struct JitKernel {
     StripPlan strip;
     // resident CTAs per SM of fn_batch by rows per thread (0: not asked yet)
     mutable std::array<std::atomic<int>, 25> per_sm{};
-    // the group's images: halo, and whether it is an external input
+    // the group's images: halo, and whether every cell in the image may be read
+    // without a test (external inputs are read as stored, but global operators
+    // keep to the valid region)
     int n_buf = 0;
     std::array<int, HVX_JIT_MAX_BUF> halo{};
-    std::array<bool, HVX_JIT_MAX_BUF> is_in{};
+    std::array<bool, HVX_JIT_MAX_BUF> whole{};
 };
 
 namespace {
@@ -1646,8 +1648,8 @@ bool jit_available() { return nvrtc().ok; }
 namespace {
 
 // Interior tiles and grid of a launch: every image's cells of an interior
-// tile grown by its halo lie in its valid region (external inputs: in the
-// image; they are read as stored).  p.rows = 0 is the tile form.  Returns the
+// tile grown by its halo lie in its valid region (JitKernel::whole: in the
+// image).  p.rows = 0 is the tile form.  Returns the
 // bytes of shared memory.
 int set_tiles(const JitKernel& k, HvxJitParams& p, unsigned* gx, unsigned* gy) {
     const int tw = p.rows ? STRIP_TW : k.tw, th = p.rows ? 8 * p.rows : k.th;
@@ -1657,7 +1659,7 @@ int set_tiles(const JitKernel& k, HvxJitParams& p, unsigned* gx, unsigned* gy) {
     for (int b = 0; b < k.n_buf; ++b) {
         const int h = k.halo[b];
         int r[4] = {0, 0, p.W, p.H};
-        if (!k.is_in[b])
+        if (!k.whole[b])
             for (int i = 0; i < 4; ++i) r[i] = p.valid[b][i];
         ix0 = std::max(ix0, ceil_div(r[0] + h, tw));
         iy0 = std::max(iy0, ceil_div(r[1] + h, th));
@@ -1810,8 +1812,10 @@ JitKernel* find_kernel(const GenericDesc& d, const std::vector<std::string>& use
         slot->n_buf = d.n_buf;
         for (int b = 0; b < d.n_buf; ++b) {
             slot->halo[b] = d.buf[b].halo;
-            slot->is_in[b] = em.ext_in[b] >= 0;
+            slot->whole[b] = em.ext_in[b] >= 0;
         }
+        for (int s = 0; s < d.n_stage; ++s)
+            if (op_is_global(d.st[s].op)) slot->whole[d.st[s].in[0]] = false;
         compile(*slot);
         if (!slot->compiled && slot->strips) {  // the tile form instead
             if (std::getenv("HVX_CODEGEN_VERBOSE"))
