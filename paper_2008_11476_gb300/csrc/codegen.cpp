@@ -1690,9 +1690,10 @@ int strip_ctas_per_sm(const JitKernel& k, int rows) {
 // are resident at a time, so that each commits one partial result.
 int reduction_ctas(const JitKernel& k, const HvxJitParams& p, long long tiles, long long all,
                    int num_sms) {
+    static_assert(STRIP_TW == 128, "strip_cta_limit's tiles");  // (of 8 x 3 rows at least)
     const long long slots = (long long)strip_ctas_per_sm(k, p.rows) * num_sms;
     const long long share = (slots * tiles + all - 1) / all;
-    return (int)std::max(1ll, std::min({tiles, share, (long long)STRIP_MAX_CTAS}));
+    return (int)std::max(1ll, std::min({tiles, share, (long long)strip_cta_limit(p.W, p.H)}));
 }
 
 // Tensor maps of the inputs that the launch's form stages by TMA.
@@ -1768,7 +1769,7 @@ std::string shape_key(const GenericDesc& d, const std::vector<std::string>& user
         c.in[e].ptr = c.out[e].ptr = nullptr;
         c.in[e].pitch = c.out[e].pitch = 0;
     }
-    for (int k = 0; k < c.n_stage; ++k) c.st[k].res = c.st[k].mirror = nullptr;
+    for (int k = 0; k < c.n_stage; ++k) c.st[k].res = c.st[k].mirror = c.st[k].scratch = nullptr;
     std::string key(reinterpret_cast<const char*>(&c), sizeof(c));
     key += std::to_string(device);
     for (const char* n : {"HVX_CODEGEN_TMA", "HVX_CODEGEN_ROWS", "HVX_CODEGEN_COLS",
@@ -1865,6 +1866,7 @@ bool jit_prepare(const GenericDesc& d, const std::vector<std::string>& user_code
         if (op_is_global(d.st[k].op)) {
             if (nres >= HVX_JIT_MAX_RES) return false;
             p.mirror[nres] = d.st[k].mirror;
+            p.scratch[nres] = d.st[k].scratch;
             p.res[nres++] = d.st[k].res;
         }
     int num_sms = 152;

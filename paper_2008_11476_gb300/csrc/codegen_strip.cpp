@@ -821,10 +821,9 @@ struct StripEmitter {
     static const char* reduction_prelude() {
         return R"STRIP(
 // ---- global operators: per-thread totals over all tiles of a CTA, one partial
-// result per CTA, combined by the last CTA to finish.  A result block is
-// followed by its scratch (16-byte aligned): a counter of finished CTAs (used
-// in the first block), then sums, per-CTA extrema or bins; the last CTA leaves
-// counter, sums and bins at zero for the next launch.  Against atomics per warp
+// result per CTA, combined by the last CTA to finish.  Scratch of each: a counter
+// of finished CTAs (the first one's is used), then sums, per-CTA extrema or bins;
+// the last CTA leaves counter, sums and bins at zero for the next launch.  Against atomics per warp
 // and tile on one result word (compare-and-swap for the counts): luma of a
 // 3840x2160 UYVY frame with MeanStdDev, MinMaxLoc and a 256-bin Histogram 1110 ->
 // 23.7 us (cold L2). ----
@@ -984,11 +983,6 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
 )STRIP";
     }
 
-    // Byte offset of a global operator's scratch counter in its result block.
-    int scratch_at(int k) const {
-        return (int)((global_result_bytes(d.st[k].op, d.st[k].i0) + 15) & ~15ull);
-    }
-
     // The kernels of a group with global operators: CTA c of p.ctas works on
     // the image's tiles c, c + p.ctas, ..
     void emit_reduction_kernels(const std::string& bounds) {
@@ -1037,8 +1031,7 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
         for (size_t j = 0; j < globals.size(); ++j) {
             const int k = globals[j];
             const std::string K = std::to_string(k),
-                              scr = "((unsigned char*)p.res[" + std::to_string(j) + "] + " +
-                                    std::to_string(scratch_at(k) + 16) + ")";
+                              scr = "((unsigned char*)p.scratch[" + std::to_string(j) + "] + 16)";
             if (d.st[k].op == OP_MEANSTD) {
                 o << "  hvx_sum_warp(acc.g" << K << ");\n"
                   << "  if ((threadIdx.x & 31) == 0) s" << K << "[threadIdx.x >> 5] = acc.g" << K << ";\n"
@@ -1065,8 +1058,7 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
         }
         // (the barrier orders the CTA's writes before thread 0's cumulative fence)
         o << "  __syncthreads();\n"
-          << "  unsigned* const done = (unsigned*)((unsigned char*)p.res[0] + " << scratch_at(globals[0])
-          << ");\n"
+          << "  unsigned* const done = (unsigned*)p.scratch[0];\n"
           << "  if (threadIdx.x == 0) {\n    __threadfence();\n"
           << "    last = atomicAdd(done, 1u) == (unsigned)p.ctas - 1u;\n  }\n"
           << "  __syncthreads();\n"
@@ -1076,8 +1068,7 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
             const int k = globals[j];
             const std::string res = "p.res[" + std::to_string(j) + "]",
                               mir = "p.mirror[" + std::to_string(j) + "]",
-                              scr = "((unsigned char*)" + res + " + " +
-                                    std::to_string(scratch_at(k) + 16) + ")";
+                              scr = "((unsigned char*)p.scratch[" + std::to_string(j) + "] + 16)";
             if (d.st[k].op == OP_MEANSTD) {
                 o << "  if (threadIdx.x < 3) {\n    const unsigned long long v = atomicExch((unsigned long "
                      "long*)"
@@ -1086,10 +1077,10 @@ __device__ __forceinline__ void hvx_mm_result(unsigned long long* r, const HvxMi
                   << ")[threadIdx.x] = v;\n  }\n";
             } else if (d.st[k].op == OP_MINMAX) {
                 o << "  {\n    HvxMinMaxAcc a;\n    hvx_mm_init(a);\n"
-                  << "    const int* const q = (const int*)" << scr << ";\n"
+                  << "    const volatile int* const q = (const volatile int*)" << scr << ";\n"
                   << "    for (int i = threadIdx.x; i < p.ctas; i += " << STRIP_THREADS << ")\n"
-                  << "      hvx_mm_merge(a, __ldcg(q + 6 * i), __ldcg(q + 6 * i + 2), __ldcg(q + 6 * i + 4), "
-                     "__ldcg(q + 6 * i + 1), __ldcg(q + 6 * i + 3), __ldcg(q + 6 * i + 5));\n"
+                  << "      hvx_mm_merge(a, q[6 * i], q[6 * i + 2], q[6 * i + 4], q[6 * i + 1], "
+                     "q[6 * i + 3], q[6 * i + 5]);\n"
                   << "    hvx_mm_block<" << warps << ">(a, smm);\n"
                   << "    if (threadIdx.x == 0) {\n      hvx_mm_result((unsigned long long*)" << res
                   << ", a);\n      if (" << mir << ") hvx_mm_result((unsigned long long*)" << mir

@@ -183,7 +183,10 @@ struct Node {
     int border = HVX_BORDER_REPLICATE;
     int cval = 0;
     int rounding = HVX_ROUND_TO_ZERO;
-    void* d_aux = nullptr;  // EqualizeHist: its 256-bin device histogram
+    // device memory kept for the node's kernels: EqualizeHist's bins, counter and
+    // mapping, a global operator's scratch
+    void* d_aux = nullptr;
+    uint64_t aux_bytes = 0;
     // set by verification
     uint32_t live_mask = 0;
     int group = -1;

@@ -26,6 +26,7 @@ struct HvxJitParams {
     unsigned long long out_pitch[HVX_JIT_MAX_EXT];
     void* res[HVX_JIT_MAX_RES];     // result blocks of the group's global operators
     void* mirror[HVX_JIT_MAX_RES];  // strip form: host copies of the results (may be null)
+    void* scratch[HVX_JIT_MAX_RES]; // strip form: CTA counter and partial results
     int* err;                       // error word (a bounded wait that ran out)
     int rows;                       // strip form: output rows per thread (tiles of 128 x 8 rows)
     int ctas;                       // strip form with global operators: CTAs of this image

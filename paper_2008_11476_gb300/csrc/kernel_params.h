@@ -61,14 +61,20 @@ HVX_HD inline bool op_is_global(int kind) {
 HVX_HD inline unsigned long long global_result_bytes(int kind, int bins) {
     return kind == OP_MEANSTD ? 24ull : kind == OP_MINMAX ? 32ull : 4ull * (unsigned long long)bins;
 }
-// A result block ends with the scratch of the strip kernels (codegen_strip.cpp),
-// 16-byte aligned: a counter of finished CTAs (16 bytes), then three 64-bit
-// sums, the extrema of up to STRIP_MAX_CTAS CTAs (24 bytes each), or the bins.
+// Scratch of a global operator's strip kernels (codegen_strip.cpp): a counter of
+// finished CTAs (16 bytes), then three 64-bit sums, the extrema of every CTA (24
+// bytes each), or the bins.  CTAs of an image: at most one per smallest tile (128
+// x 24 pixels), and STRIP_MAX_CTAS.  It is not part of the result block, which
+// counts against the context's memory budget.
 constexpr int STRIP_MAX_CTAS = 1024;
-HVX_HD inline unsigned long long global_block_bytes(int kind, int bins) {
-    return ((global_result_bytes(kind, bins) + 15) & ~15ull) + 16 +
-           (kind == OP_MEANSTD ? 24ull : kind == OP_MINMAX ? 24ull * STRIP_MAX_CTAS
-                                                           : 4ull * (unsigned long long)bins);
+HVX_HD inline int strip_cta_limit(int W, int H) {
+    const long long tiles = (long long)((W + 127) / 128) * ((H + 23) / 24);
+    return tiles < STRIP_MAX_CTAS ? (int)tiles : STRIP_MAX_CTAS;
+}
+HVX_HD inline unsigned long long global_scratch_bytes(int kind, int bins, int W, int H) {
+    return 16 + (kind == OP_MEANSTD ? 24ull
+                 : kind == OP_MINMAX ? 24ull * (unsigned long long)strip_cta_limit(W, H)
+                                     : 4ull * (unsigned long long)bins);
 }
 HVX_HD inline int global_result_fill(int kind) { return kind == OP_MINMAX ? 0xFF : 0; }
 
@@ -112,7 +118,8 @@ struct GenStage {
     float f0, f1;      // F32 thresholds
     int64_t k0, k1;    // integer thresholds, or kn / kd of the Harris response
     void* res;         // global operators: device result block (out is -1)
-    void* mirror;      // ... and its host copy that the device writes (may be null)
+    void* mirror;      // ... its host copy that the device writes (may be null)
+    void* scratch;     // ... and the strip kernels' scratch
 };
 
 struct GenExt {

@@ -619,6 +619,7 @@ hvx_status build_generic(Plan& P, Group& G) {
         st.out = op.out->is_result ? -1 : buf[op.out];
         st.res = op.out->is_result ? op.out->dev : nullptr;
         st.mirror = op.out->is_result ? op.out->mirror_dev : nullptr;
+        st.scratch = op.out->is_result ? op.node->d_aux : nullptr;
         st.rx = op.rx;
         st.ry = op.ry;
         st.rounding = op.node->rounding;
@@ -763,14 +764,14 @@ hvx_status check_device_error(Context* ctx) {
 }
 
 // Device result blocks of global operators (kept with the result image for
-// the life of the graph) and EqualizeHist's histogram; *clearing: a new block's
+// the life of the graph), their scratch and EqualizeHist's (kept with the node,
+// not counted against the memory budget); *clearing: a new block's
 // memset has been queued on the legacy stream.
 hvx_status alloc_result_blocks(Plan& P, Context* ctx, bool* clearing) {
     for (int i : P.order) {
         Op& op = P.ops[i];
         if (op_is_global(op.kind)) {
-            const uint64_t res = global_result_bytes(op.kind, op.node->p.hist_bins);
-            const uint64_t n = global_block_bytes(op.kind, op.node->p.hist_bins);
+            const uint64_t n = global_result_bytes(op.kind, op.node->p.hist_bins);
             if (op.out->dev && op.out->bytes != n) {
                 ctx->pool.free(op.out->dev);
                 op.out->dev = nullptr;
@@ -779,8 +780,7 @@ hvx_status alloc_result_blocks(Plan& P, Context* ctx, bool* clearing) {
                 void* p = nullptr;
                 hvx_status st = ctx->pool.alloc(n, &p);
                 if (st != HVX_SUCCESS) return st;
-                cudaError_t e = cudaMemset(p, 0, n);
-                if (e == cudaSuccess) e = cudaMemset(p, global_result_fill(op.kind), res);
+                const cudaError_t e = cudaMemset(p, global_result_fill(op.kind), n);
                 if (e != cudaSuccess) {
                     cudaGetLastError();
                     ctx->pool.free(p);
@@ -791,24 +791,31 @@ hvx_status alloc_result_blocks(Plan& P, Context* ctx, bool* clearing) {
                 op.out->bytes = n;
                 *clearing = true;
             }
-            if (!op.out->mirror && ctx->host.alloc(res, &op.out->mirror, &op.out->mirror_dev)) {
-                op.out->mirror_bytes = res;
-                std::memset(op.out->mirror, global_result_fill(op.kind), res);
+            if (!op.out->mirror && ctx->host.alloc(n, &op.out->mirror, &op.out->mirror_dev)) {
+                op.out->mirror_bytes = n;
+                std::memset(op.out->mirror, global_result_fill(op.kind), n);
             }
         }
-        if (op.kind == OP_EQHIST && !op.node->d_aux) {
+        const uint64_t aux =
+            op.kind == OP_EQHIST ? EQHIST_BYTES
+            : op_is_global(op.kind)
+                ? global_scratch_bytes(op.kind, op.node->p.hist_bins, (int)op.in[0]->w, (int)op.in[0]->h)
+                : 0;
+        if (aux > op.node->aux_bytes) {
             void* p = nullptr;
-            if (cudaMalloc(&p, EQHIST_BYTES) != cudaSuccess) {
+            if (cudaMalloc(&p, aux) != cudaSuccess) {
                 cudaGetLastError();
                 return HVX_ERROR_NO_MEMORY;
             }
-            const cudaError_t e = cudaMemset(p, 0, EQHIST_BYTES);
+            const cudaError_t e = cudaMemset(p, 0, aux);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 cudaFree(p);
                 return cuda_status(e);
             }
+            if (op.node->d_aux) cudaFree(op.node->d_aux);
             op.node->d_aux = p;
+            op.node->aux_bytes = aux;
             *clearing = true;
         }
     }

@@ -145,3 +145,53 @@ def test_blocks_of_a_released_graph_are_idle(ctx):
         H.hvxProcessGraph(g)
         check_group(nodes, ref)
         H.hvxReleaseGraph(g)
+
+
+@pytest.mark.parametrize("w,h", [(7, 5), (1920, 1080)])
+def test_only_results_count_against_the_budget(w, h):
+    """256 bytes (the pool's step) for MeanStdDev and MinMaxLoc, 1024 for 256
+    bins, whatever the image's size: a budget of just that verifies."""
+    c = H.hvxCreateContext()
+    try:
+        src = PG.upload(c, synth.rects_noise(w, h, 1), H.HVX_DF_U8)
+        used = H.hvxGetContextMemoryUsage(c)
+        g = H.hvxCreateGraph(c)
+        H.hvxMeanStdDevNode(g, src)
+        mm = H.hvxMinMaxLocNode(g, src)
+        H.hvxHistogramNode(g, src, 256, 0, 256)
+        H.hvxSetContextMemoryBudget(c, used + 256 + 256 + 1024)
+        H.hvxVerifyGraph(g)
+        assert H.hvxGetContextMemoryUsage(c) == used + 256 + 256 + 1024
+        H.hvxProcessGraph(g)
+        img = PG.download(src)
+        assert H.hvxGetNodeResult(mm, H.HvxMinMaxLoc()).max_count == (img == img.max()).sum()
+    finally:
+        H.hvxReleaseContext(c)
+
+
+def test_minmax_of_every_tile_count():
+    """The extrema's scratch holds one entry per CTA: sizes around the limits of
+    one tile, of tiles per CTA and of 1024 CTAs, alone and batched."""
+    c = H.hvxCreateContext()
+    try:
+        graphs = []
+        for w, h in [(1, 1), (128, 24), (129, 25), (1, 32768), (32768, 1), (4096, 2160)]:
+            img = synth.uniform_u8(w, h, w + h)
+            g = H.hvxCreateGraph(c)
+            mm = H.hvxMinMaxLocNode(g, PG.upload(c, img, H.HVX_DF_U8))
+            H.hvxVerifyGraph(g)
+            graphs.append((g, mm, img))
+        for batch in (False, True):
+            if batch:
+                H.hvxProcessGraphBatch([g for g, _, _ in graphs])
+            else:
+                for g, _, _ in graphs:
+                    H.hvxScheduleGraph(g)
+            H.hvxWaitBatch(c)
+            for _, mm, img in graphs:
+                r = H.hvxGetNodeResult(mm, H.HvxMinMaxLoc())
+                assert (r.min, r.max, r.min_count, r.max_count) == (
+                    img.min(), img.max(), (img == img.min()).sum(), (img == img.max()).sum())
+                assert img.argmin() == r.min_y * img.shape[1] + r.min_x
+    finally:
+        H.hvxReleaseContext(c)
