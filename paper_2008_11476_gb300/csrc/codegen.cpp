@@ -531,10 +531,12 @@ struct Emitter {
                 if (slot[t].def <= slot[s].last && slot[s].def <= slot[t].last)
                     busy.push_back({slot[t].off, slot[t].off + slot_words(t)});
             std::sort(busy.begin(), busy.end());
+            // a TMA destination starts on a 128-byte boundary
+            const int align = s < d.n_buf && tma_slot(s) ? 32 : 1;
             int off = 0;
             for (const auto& iv : busy) {
                 if (off + n <= iv.first) break;
-                off = std::max(off, iv.second);
+                off = std::max(off, (iv.second + align - 1) / align * align);
             }
             slot[s].off = off;
             placed.push_back(s);
@@ -847,6 +849,8 @@ struct Emitter {
           << "    if (threadIdx.x == 0) hvx_mbar_init(bar);\n"
           << "    __syncthreads();\n"
           << "    if (threadIdx.x == 0) {\n"
+          << "      // (the slots may have held other images)\n"
+          << "      asm volatile(\"fence.proxy.async.shared::cta;\" ::: \"memory\");\n"
           << "      hvx_expect_tx(bar, " << bytes << "u);\n";
         for (int b : T) {
             const int e = ext_in[b];
@@ -1536,7 +1540,7 @@ struct Emitter {
           << "  // previous grid on the stream has completed\n"
           << "  asm volatile(\"griddepcontrol.launch_dependents;\");\n"
           << "  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");\n"
-          << "  extern __shared__ __align__(16) int smem[];\n"
+          << "  extern __shared__ __align__(128) int smem[];  // (bins may lie before it)\n"
           << "  const int tx = blockIdx.x, ty = blockIdx.y;\n"
           << "  if (tx >= p.ix0 && tx <= p.ix1 && ty >= p.iy0 && ty <= p.iy1)\n"
           << "    hvx_tile<false, false>(p, smem, tx * " << tw << ", ty * " << th << ");\n"
@@ -1548,7 +1552,7 @@ struct Emitter {
           << "extern \"C\" __global__ void __launch_bounds__(" << kThreads << min_blocks()
           << ") hvx_generated_batch(const HvxJitParams* __restrict__ ps, const int* __restrict__ "
              "tile_start, int n) {\n"
-          << "  extern __shared__ __align__(16) int smem[];\n"
+          << "  extern __shared__ __align__(128) int smem[];  // (bins may lie before it)\n"
           << "  const int t = blockIdx.x;\n"
           << "  int lo = 0, hi = n - 1;\n"
           << "  while (lo < hi) {\n"
