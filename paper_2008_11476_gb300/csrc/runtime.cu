@@ -842,14 +842,19 @@ hvx_status prepare_launches(Graph* g) {
         hvx_status st = alloc_results(P, ctx);
         if (st != HVX_SUCCESS) return st;
     }
-    // HVX_CODEGEN_ONLY: generated kernels in place of the hand-written ones
-    const bool hand = g->codegen != HVX_CODEGEN_ONLY;
     const bool must_gen = g->codegen == HVX_CODEGEN_REQUIRE || g->codegen == HVX_CODEGEN_ONLY;
     P.stateful = false;
     for (int i : P.order)
         P.stateful = P.stateful || op_is_global(P.ops[i].kind) || P.ops[i].kind == OP_EQHIST;
     for (Group& G : P.groups) {
         G.ext_bytes = G.mem_bytes = 0;
+        // HVX_CODEGEN_ONLY: generated kernels in place of the hand-written ones.  Those
+        // place their border tiles by the image's edges, so an input whose valid
+        // region is smaller (stored by another group) takes the general kernels.
+        bool hand = g->codegen != HVX_CODEGEN_ONLY;
+        for (const Image* im : G.inputs)
+            hand = hand && im->valid.x0 == 0 && im->valid.y0 == 0 && im->valid.x1 == (int)im->w &&
+                   im->valid.y1 == (int)im->h;
         for (Image* im : G.inputs) {
             G.mem_bytes += image_bytes(im);
             if (!im->is_virtual) G.ext_bytes += image_bytes(im);
