@@ -1052,10 +1052,12 @@ struct BatchCache {
 
 // A batch's tables to the device, complete on return (its launches read them
 // without waiting for the stream's previous work, on any stream).  By the
-// internal stream: the legacy one is closed while a blocking stream is captured.
+// internal stream where there is one: the legacy one is closed while a blocking
+// stream is captured.
 cudaError_t upload(BatchCache* bc, void* dev, const void* host, size_t bytes) {
-    const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, bc->trial);
-    return e == cudaSuccess ? cudaStreamSynchronize(bc->trial) : e;
+    const cudaStream_t s = bc->trial ? bc->trial : cudaStreamLegacy;
+    const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
 // While it lives, the thread may allocate although a stream is being captured.
@@ -1560,7 +1562,8 @@ hvx_status process_batch(Context* ctx, Graph* const* gs, int n, cudaStream_t s) 
             bc->entries.erase(oldest);
         }
         RelaxedCapture relaxed;
-        if (!bc->trial) {
+        // (creating a stream takes 10 us of a first call)
+        if (!bc->trial && (same || capturing)) {
             const cudaError_t e = cudaStreamCreateWithFlags(&bc->trial, cudaStreamNonBlocking);
             if (e != cudaSuccess) return cuda_status(e);
         }
