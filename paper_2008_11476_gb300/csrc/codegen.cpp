@@ -20,9 +20,9 @@
 //     template.
 // Kernels are cached by source text, so graphs of the same shape share one.
 // A group whose images fit 16-bit lanes runs the strip form instead
-// (codegen_strip.cpp, faster at every size measured); the tile form stays for
-// S32 / F32 images, 64-bit user operators, global operators and sums beyond 16
-// bits, and for the tuning knobs that ask for one of its variants.
+// (codegen_strip.cpp, faster at every size measured), global operators
+// included; the tile form stays for S32 / F32 images, user operators and sums
+// beyond 16 bits, and for the tuning knobs that ask for one of its variants.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <dlfcn.h>
@@ -1722,12 +1722,15 @@ bool set_maps(const JitKernel& k, HvxJitParams& p) {
 // its R rows and the prologue steps before them; the launch takes waves of the
 // CTAs that are resident at a time (registers, and boxes that grow with R), the
 // last one partly filled.  Minimising max(1, waves + 1/2) (R + 0.3 prologue +
-// 1) comes within 0.4 % of the best R in the mean and 5.5 % at worst over 44
-// measured points (FChain, Unsharp, Laplacian and a morphology graph; 64x48 to
-// 3840x2160; 1 to 16 frames; R = 3 .. 24): small launches want R = 3 (1080p
-// Unsharp frame: 5.0 us, 11.8 at R = 15), 16 x 1080p FChain R = 15 (57 us, 107
-// at R = 3), 16 x 1080p Unsharp R = 9 (25 us, 41 and 40 at R = 3 and 24), all
-// before border tiles filled only the ring that is read (FChain now 52 us).
+// 1) comes within 4 % of the best R in the mean over 47 measured points (FChain,
+// Unsharp, Laplacian, a morphology graph, and luma with three global operators;
+// 64x48 to 3840x2160; 1 to 16 frames; every R): 0.1 % for the morphology graph,
+// 1-2 % for FChain and the global operators, 7 and 9 % for Unsharp and Laplacian,
+// whose short groups want more rows than the model gives them where about one
+// wave is launched (4 x 1080p: Laplacian 8.0 us at the chosen R = 3, 5.5 at R =
+// 6; Unsharp 8.5 and 6.2; the worst points).  Small launches want R = 3 (1080p
+// Unsharp frame: 3.2 us, 4.0 at R = 15), 16 x 1080p FChain R = 15 (49 us, 99 at R
+// = 3), 16 x 1080p Unsharp R = 15 (16.5 us; R = 9 is chosen, 17.9; 33.9 at R = 3).
 // HVX_STRIP_ROWS in the environment overrides (0: the tile form).
 int strip_rows(const JitKernel& k, const int* W, const int* H, int n, int num_sms) {
     const int u = k.strip.unroll;

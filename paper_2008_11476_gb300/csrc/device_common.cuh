@@ -249,7 +249,7 @@ __device__ __forceinline__ void for_each_outside(int R, int C, int bx, int by, i
 // stencil of radius HALO reads outside the image.
 template <int HALO, class F>
 __device__ __forceinline__ void for_each_ring(int x0, int y0, int tw, int th, int W, int H, F f) {
-    const int c0 = x0 == 0 ? -HALO : x0 - HALO, c1 = min(x0 + tw, W) + HALO;
+    const int c0 = x0 - HALO, c1 = min(x0 + tw, W) + HALO;
     const int r0 = max(y0 - HALO, 0), r1 = min(y0 + th + HALO, H);  // rows inside the image
 #pragma unroll
     for (int k = 1; k <= HALO; ++k)

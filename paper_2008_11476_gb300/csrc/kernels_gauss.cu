@@ -338,10 +338,10 @@ cudaError_t launch_gauss(const CUtensorMap& map, const EdgeParams& p, cudaStream
     }
 }
 
-// Rows per thread of the single-image Gaussian kernel (tiles of 128 x 8R):
-// as for the edge kernel, R = 5, or R = 2 when the image has fewer 128 x 40
-// tiles than SMs (a small image then still spreads over the GPU), so that a
-// launch's latency is a few rows of work per thread.
+// Rows per thread of the single-image Gaussian and 5x5 binomial kernels (tiles
+// of 128 x 8R): R = 5, or R = 2 when the image has fewer 128 x 40 tiles than SMs
+// (a small image then still spreads over the GPU), so that a launch's latency is
+// a few rows of work per thread.
 int gauss_single_rows(int W, int H, int num_sms) {
     const long long tiles5 = (long long)((W + TW - 1) / TW) * ((H + 39) / 40);
     return tiles5 >= (num_sms > 0 ? num_sms : 152) ? 5 : 2;

@@ -8,8 +8,9 @@
 // The histogram is bound by shared-memory atomics: 8 copies of the bins, one
 // per lane modulo 8, halve the bank conflicts of one copy.  The mapping is
 // bound by the latency of its loads and the byte look-ups in shared memory.
-// 3840x2160 (cold L2, one launch each): count 16.0 -> 12.7 us, mapping 23.4 ->
-// 9.6 us against one pixel per thread step.
+// 3840x2160 (cold L2, one launch each): count 16.0 -> 11.5 us, mapping 23.4 ->
+// 7.4 us against one pixel per thread step (12.7 and 9.6 without the loads one
+// step ahead).
 #include "device_common.cuh"
 #include "launchers.h"
 
@@ -175,7 +176,7 @@ int grid_for(unsigned long long steps, int num_sms) {
 
 cudaError_t launch_eqhist(const EqHistParams& p, cudaStream_t s) {
     const unsigned long long steps = (unsigned long long)((p.W + 15) / 16) * p.H;
-    // (at least ~8 steps per thread share the count's 8 KB of bins and its commit)
+    // (about 4 steps per thread share the count's 8 KB of bins and its commit)
     cudaError_t e = launch_pdl(eqhist_count_kernel, dim3(grid_for((steps + 3) / 4, p.num_sms)),
                                dim3(kThreads), 0, s, p);
     if (e != cudaSuccess) return e;

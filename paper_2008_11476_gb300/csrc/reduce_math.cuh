@@ -4,7 +4,8 @@
 // the kernels generated for fused groups (self-contained, like
 // point_math.cuh).
 //
-// Device result blocks (zeroed / set to all ones before each launch):
+// Device result blocks (the interpreter and the tile form add to them, zeroed /
+// set to all ones before each launch; the strip form writes them whole):
 //   MeanStdDev: long long S1; unsigned long long S2, N       (zeroed)
 //   MinMaxLoc:  unsigned long long min_key, max_key,           (all ones)
 //               min_pack, max_pack

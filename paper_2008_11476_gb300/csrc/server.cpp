@@ -67,7 +67,13 @@ struct Server {
     void run();
 };
 
-// How long after the last progress the dispatcher polls without sleeping.
+// How long after the last progress the dispatcher polls without sleeping while
+// requests are in flight or queued.  With 0 / 0.02 / 0.05 / 0.1 / 0.5 / 1 ms: 32
+// requests at once 335 / 240 / 240 / 239 / 240 / 240 us; Poisson 2000 requests/s
+// p50 88 / 28 / 29 / 28 / 28 / 28 us, p99 127 / 115 / 145 / 91 / 92 / 91 us, the
+// dispatcher on its core for 2 / 4 / 5 / 5 / 5 / 5 % of the time (8 to 23 % at 10000
+// requests/s).  From 0.1 ms on nothing changes for these requests; 0.5 leaves room
+// for longer ones.
 constexpr double kBusyMs = 0.5;
 
 void Server::run() {
